@@ -21,7 +21,7 @@ constexpr int MIN_CHUNK = 32;         // fewest points per work unit
 #define RF_UNITS_PER_WARP 16
 #endif
 constexpr int UNITS_PER_WARP = RF_UNITS_PER_WARP;  // target work units per warp and iteration
-constexpr int APW = 16;               // doubles per CTA in the APS partials
+constexpr int APW = 16;               // doubles per CTA in the APS partials: 8 sums, then one int4
 constexpr int MAX_CTAS_PER_SM = 2048 / FIT_THREADS;  // bound for grid-sized scratch
 // CTAs of the persistent kernel resident per SM (register budget 65536 / (256 * n)).
 // Measured on the paper-scale frame: groups of 6 lookups at 2 CTAs per SM 312.7 G
@@ -433,19 +433,7 @@ __device__ __forceinline__ void fitness_units(const VolumeDesc &V, const float4 
     }
 }
 
-// Fixed-order sum of the chunk partials of particle i, then rho (Eq. normallh,
-// or Eq. ourlh without NORMALIZE).
-__device__ __forceinline__ void particle_total(const double *part_S, const int *part_n, int n, int n_chunks, int i,
-                                               bool coherent, double &S, int &nv)
-{
-    S = 0.0;
-    nv = 0;
-    for (int c = 0; c < n_chunks; ++c) {
-        S += coherent ? __ldcg(&part_S[(size_t)c * n + i]) : part_S[(size_t)c * n + i];
-        nv += coherent ? __ldcg(&part_n[(size_t)c * n + i]) : part_n[(size_t)c * n + i];
-    }
-}
-
+// rho of a particle's total (Eq. normallh, or Eq. ourlh without NORMALIZE).
 __device__ __forceinline__ float fitness_rho(double S, int nO, float tau, bool normalize)
 {
     if (nO <= 0)

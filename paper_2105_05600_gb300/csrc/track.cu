@@ -30,15 +30,42 @@ __global__ void __launch_bounds__(FIT_THREADS) fitness_kernel(VolumeDesc V, cons
                                    lane, w);
 }
 
-__global__ void fitness_finish_kernel(int n, int n_chunks, const double *part_S, const int *part_n, int m, float tau,
-                                      int normalize, float *rho, double *sumsq, int *nvalid)
+// Totals of the chunk partials ([chunk][particle]) and rho.  A block takes 32
+// particles, its warps every FINISH_WARPS-th chunk each, so the loads are
+// contiguous runs of 32 particles and a particle's chunks are read side by side;
+// the warps' sums meet in shared memory in a fixed order.  Bound by the latency of
+// ceil(n_chunks / 32) loads per thread, 8 in flight: one thread per particle, which
+// walked the chunks alone, took 253 us for 256 particles x 600 chunks and 70 us for
+// 20,000 x 63.
+constexpr int FINISH_WARPS = 32;
+__global__ void __launch_bounds__(FINISH_WARPS * 32) fitness_finish_kernel(int n, int n_chunks, const double *part_S,
+                                                                           const int *part_n, int m, float tau,
+                                                                           int normalize, float *rho, double *sumsq,
+                                                                           int *nvalid)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n)
+    __shared__ double s_S[FINISH_WARPS][32];
+    __shared__ int s_n[FINISH_WARPS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    double S = 0.0;
+    int nv = 0;
+    if (i < n) {
+#pragma unroll 8
+        for (int c = w; c < n_chunks; c += FINISH_WARPS) {
+            S += part_S[(size_t)c * n + i];
+            nv += part_n[(size_t)c * n + i];
+        }
+    }
+    s_S[w][lane] = S;
+    s_n[w][lane] = nv;
+    __syncthreads();
+    if (w != 0 || i >= n)
         return;
-    double S;
-    int nv;
-    particle_total(part_S, part_n, n, n_chunks, i, false, S, nv);
+    const int q_end = min(FINISH_WARPS, n_chunks);
+    for (int q = 1; q < q_end; ++q) {
+        S += s_S[q][lane];
+        nv += s_n[q][lane];
+    }
     rho[i] = fitness_rho(S, m, tau, normalize != 0);
     if (sumsq)
         sumsq[i] = S;
@@ -177,7 +204,7 @@ rf_status fitness_eval(rf_volume v, const float *points_dev, int m, const float 
     fp.right_mult = (p->flags & RF_RIGHT_MULT) != 0;
     fn<<<grid, FIT_THREADS, smem, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
     RF_CUDA(cudaGetLastError());
-    fitness_finish_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
+    fitness_finish_kernel<<<(n + 31) / 32, FINISH_WARPS * 32, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
                                                           (p->flags & RF_NORMALIZE) != 0, rho_dev, sumsq_dev,
                                                           nvalid_dev);
     RF_CUDA(cudaGetLastError());
@@ -262,7 +289,7 @@ extern "C" rf_status fitness_eval_noalloc(rf_volume v, const float *points_dev, 
     fp.right_mult = (p->flags & RF_RIGHT_MULT) != 0;
     fn<<<grid, FIT_THREADS, smem, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
     RF_CUDA(cudaGetLastError());
-    fitness_finish_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
+    fitness_finish_kernel<<<(n + 31) / 32, FINISH_WARPS * 32, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
                                                           (p->flags & RF_NORMALIZE) != 0, rho_dev, sumsq_dev,
                                                           nvalid_dev);
     RF_CUDA(cudaGetLastError());
