@@ -72,12 +72,13 @@ struct LaunchScratch {
     int *unit_ctr = nullptr;
     int *block_counts = nullptr;
     double *aps = nullptr;
+    static size_t cleared_bytes() { return sizeof(GridSync) + sizeof(int) * RF_MAX_ITERS; }  // gs and unit_ctr
     rf_status alloc()
     {
         const size_t max_grid = (size_t)MAX_CTAS_PER_SM * sm_count();
-        cudaError_t e = cudaMalloc(&gs, sizeof(GridSync));
+        cudaError_t e = cudaMalloc(&gs, cleared_bytes());
         if (e == cudaSuccess)
-            e = cudaMalloc(&unit_ctr, sizeof(int) * RF_MAX_ITERS);
+            unit_ctr = reinterpret_cast<int *>(gs + 1);
         if (e == cudaSuccess)
             e = cudaMalloc(&block_counts, sizeof(int) * MAX_BATCH * max_grid);
         if (e == cudaSuccess)
@@ -89,7 +90,6 @@ struct LaunchScratch {
     void release()
     {
         cudaFree(gs);
-        cudaFree(unit_ctr);
         cudaFree(block_counts);
         cudaFree(aps);
         gs = nullptr;
@@ -213,8 +213,8 @@ static rf_status fill_problem(rf_tracker tr, const float *depth, const float *pr
     return RF_OK;
 }
 
-// Enqueue one persistent launch for B prepared problems: resets of the barrier,
-// counters, statuses and stats, then the cooperative kernel.  Capturable.
+// Enqueue one persistent launch for B prepared problems: reset of the barrier and the
+// unit counters, then the cooperative kernel (which clears statuses and stats).  Capturable.
 static rf_status launch_batch(BatchParams &P, const LaunchScratch &ls, int dtype, int mode, int ctas_per_sm,
                               int group, int debug_skip, cudaStream_t s)
 {
@@ -229,14 +229,9 @@ static rf_status launch_batch(BatchParams &P, const LaunchScratch &ls, int dtype
     P.block_counts = ls.block_counts;
     P.aps = ls.aps;
     P.k_max_all = 0;
-    for (int p = 0; p < P.B; ++p) {
+    for (int p = 0; p < P.B; ++p)
         P.k_max_all = std::max(P.k_max_all, P.prob[p].k_max);
-        RF_CUDA(cudaMemsetAsync(P.prob[p].status, 0, sizeof(int), s));
-        if (P.prob[p].stats)
-            RF_CUDA(cudaMemsetAsync(P.prob[p].stats, 0, sizeof(rf_frame_stats), s));
-    }
-    RF_CUDA(cudaMemsetAsync(ls.gs, 0, sizeof(GridSync), s));
-    RF_CUDA(cudaMemsetAsync(ls.unit_ctr, 0, sizeof(int) * RF_MAX_ITERS, s));
+    RF_CUDA(cudaMemsetAsync(ls.gs, 0, LaunchScratch::cleared_bytes(), s));
     if (debug_skip) {
         set_int_kernel<<<1, 1, 0, s>>>(&ls.gs->skip, 1);
         RF_CUDA(cudaGetLastError());

@@ -49,8 +49,7 @@ struct ProblemDesc {
 };
 
 struct GridSync {
-    unsigned int count;
-    unsigned int gen;
+    unsigned int count;  // CTAs that have arrived, over all barriers of the launch
     int abort;
     int skip;  // test hook: block 0 leaves at the first barrier without arriving
 };
@@ -60,59 +59,64 @@ struct BatchParams {
     int B;
     int k_max_all;
     int work_warps;
-    GridSync *gs;
-    int *unit_ctr;      // [RF_MAX_ITERS], zero at launch
+    GridSync *gs;       // gs and unit_ctr are one allocation, zero at launch
+    int *unit_ctr;      // [RF_MAX_ITERS]
     int *block_counts;  // [grid][MAX_BATCH]
     double *aps;        // [grid][MAX_BATCH][APW]
     long long timeout_ns;
 };
 
 // ------------------------------------------------------------------ grid barrier
-// Sense-reversing counter barrier over all CTAs of the cooperative launch.  Every
-// wait is bounded: after timeout_ns the CTA sets `abort`, marks every sequence's
-// status RF_ERR_TIMEOUT and returns false; waiters that see `abort` return false.
-static __device__ bool grid_barrier(const BatchParams &P)
+// Counter barrier over all CTAs of the cooperative launch.  `count` only grows: the
+// n-th barrier is open once it reaches n x gridDim, so an arrival is one release
+// increment and a wait is one polled word -- no reset, no second flag to pass on
+// and no back-off sleep (304 CTAs of a GB300, all arriving together: 1.5 to 2.1 us,
+// against 2.3 to 2.9 us for a sense-reversing counter with a generation word).  Every
+// wait is bounded: after timeout_ns the CTA sets
+// `abort`, marks every sequence's status RF_ERR_TIMEOUT and returns false; waiters
+// that see `abort` return false.  `n` counts this CTA's barriers (thread 0).
+static __device__ bool grid_barrier(const BatchParams &P, unsigned int &n)
 {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         GridSync *gs = P.gs;
         int ok = 1;
-        volatile unsigned int *vgen = &gs->gen;
         volatile int *vabort = &gs->abort;
         if (*vabort) {
             ok = 0;
         } else if (gs->skip && blockIdx.x == 0) {
             ok = 0;  // leave without arriving
         } else {
-            const unsigned int g = *vgen;
-            __threadfence();
-            const unsigned int prev = atomicAdd(&gs->count, 1u);
-            if (prev == gridDim.x - 1) {
-                atomicExch(&gs->count, 0u);
-                __threadfence();
-                atomicAdd(&gs->gen, 1u);
-            } else {
-                const long long t0 = global_ns();
-                unsigned int ns = 32;
-                while (*vgen == g) {
-                    if (*vabort) {
-                        ok = 0;
-                        break;
-                    }
-                    if (global_ns() - t0 > P.timeout_ns) {
-                        atomicExch(&gs->abort, 1);
-                        for (int p = 0; p < P.B; ++p)
-                            atomicCAS(P.prob[p].status, 0, RF_ERR_TIMEOUT);
-                        ok = 0;
-                        break;
-                    }
-                    __nanosleep(ns);
-                    if (ns < 256)
-                        ns <<= 1;
+            const unsigned int target = ++n * gridDim.x;
+            // release: the CTA's writes, ordered before thread 0 by __syncthreads, are
+            // visible to whoever acquires a later value of count
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gs->count) : "memory");
+            // relaxed polls and one fence at the end: an acquire load drops the SM's L1, which
+            // the other CTA may still be scoring from
+            long long t0 = 0;
+            for (unsigned int polls = 0;; ++polls) {
+                unsigned int c;
+                asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&gs->count) : "memory");
+                if (c >= target)
+                    break;
+                if ((polls & 15u) != 0u)
+                    continue;
+                if (polls == 0)
+                    t0 = global_ns();
+                if (*vabort) {
+                    ok = 0;
+                    break;
+                }
+                if (global_ns() - t0 > P.timeout_ns) {
+                    atomicExch(&gs->abort, 1);
+                    for (int p = 0; p < P.B; ++p)
+                        atomicCAS(P.prob[p].status, 0, RF_ERR_TIMEOUT);
+                    ok = 0;
+                    break;
                 }
             }
-            __threadfence();
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
         }
         s_ok = ok;
     }
@@ -154,26 +158,23 @@ __device__ __forceinline__ void merge_max(float &rm, int &am, float &rs, float o
     rs = n2;
 }
 
-// Total over the chunk partials of particle i (stored [particle][chunk], coherent
-// loads): lane l sums chunks l, l + 32, ... and a fixed butterfly combines the
-// lanes; lane 0's result is the total.  The order is fixed, so the same particle
-// always gets the same value.
-__device__ __forceinline__ void warp_particle_total(const double *part_S, const int *part_n, int n_chunks, int i,
-                                                    int lane, double &S, int &nv)
+// Sums of eight values over a warp: lane l < 8 returns the total of v[l].  Halving
+// the values with every exchange takes 9 FP64 additions where eight butterflies
+// take 40 (an FP64 instruction of a warp holds the SM's FP64 unit for 16 clocks).
+__device__ __forceinline__ double warp_sum8(double v[8], int lane)
 {
-    const size_t row = (size_t)i * n_chunks;
-    double s = 0.0;
-    int c = 0;
-    for (int ch = lane; ch < n_chunks; ch += 32) {
-        s += __ldcg(&part_S[row + ch]);
-        c += __ldcg(&part_n[row + ch]);
+#pragma unroll
+    for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    S = s;
-    nv = c;
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return __shfl_sync(0xffffffffu, v[0], ((lane & 4) << 2) | ((lane & 2) << 2) | ((lane & 1) << 2));
 }
 
 // Per-sequence state, identical in every CTA (computed redundantly in a fixed order).
@@ -195,17 +196,29 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
     extern __shared__ float4 smem_pts[];
     __shared__ PState st[MAX_BATCH];
     __shared__ int warp_tot[FIT_WARPS];
-    __shared__ double red_d[FIT_WARPS][8];
-    __shared__ float red_f[FIT_WARPS][2];
-    __shared__ int red_i[FIT_WARPS][2];
-    __shared__ long long red_v[FIT_WARPS];
+    __shared__ double share_S[FIT_WARPS][32];
+    __shared__ int share_n[FIT_WARPS][32];
+    __shared__ double red_d[FIT_WARPS];
+    __shared__ float red_f[2];
+    __shared__ int red_i[3];
+    static_assert(FIT_WARPS == 8, "phase C: one warp per APS quantity");
     __shared__ int s_total_units;
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int G = gridDim.x, b = blockIdx.x;
     const int B = P.B;
+    unsigned int n_barriers = 0;
 
-    // ---- prologue: unproject the points of every level of every sequence (Eq. unproj)
+    // ---- prologue: clear the statistics and statuses (here and not by one memset each:
+    // a stream operation costs a small frame about 2 us), unproject the points of every
+    // level of every sequence (Eq. unproj)
+    for (int p = b; p < B; p += G) {
+        if (P.prob[p].stats)
+            for (int i = tid; i < (int)(sizeof(rf_frame_stats) / sizeof(int)); i += blockDim.x)
+                reinterpret_cast<int *>(P.prob[p].stats)[i] = 0;
+        if (tid == 0)
+            *P.prob[p].status = 0;
+    }
     {
         long long total = 0;
         for (int p = 0; p < B; ++p)
@@ -249,7 +262,7 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
         s.iters = 0;
         s.lookups = 0;
     }
-    if (!grid_barrier(P))
+    if (!grid_barrier(P, n_barriers))
         return;
 
     for (int k = 1; k <= P.k_max_all; ++k) {
@@ -310,7 +323,7 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 base += st[p].m_lvl;
             }
         }
-        if (!grid_barrier(P))
+        if (!grid_barrier(P, n_barriers))
             return;
         // ---- phase A': per-sequence offsets and |O_k|, then the compaction
         for (int p = w; p < B; p += FIT_WARPS) {
@@ -382,7 +395,7 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 base += st[p].m_lvl;
             }
         }
-        if (!grid_barrier(P))
+        if (!grid_barrier(P, n_barriers))
             return;
         // ---- phase B: fitness of every particle of every active sequence (Eq. normallh)
         if (tid == 0) {
@@ -441,14 +454,14 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 double S;
                 int nv;
                 fitness_lane<DT, MODE, LG>(pd.V, spts, cnt, fp, i, S, nv);
-                if (i < s.n_lvl) {  // partials stored [particle][chunk]: phase B' reads a particle's row
-                    pd.part_S[(size_t)i * s.n_chunks + ch] = S;
-                    pd.part_n[(size_t)i * s.n_chunks + ch] = nv;
+                if (i < s.n_lvl) {  // stored [chunk][particle]: a warp's partials are contiguous
+                    pd.part_S[(size_t)ch * s.n_lvl + i] = S;
+                    pd.part_n[(size_t)ch * s.n_lvl + i] = nv;
                 }
                 u = u_next;
             }
         }
-        if (!grid_barrier(P))
+        if (!grid_barrier(P, n_barriers))
             return;
         // ---- phase B': per-particle totals, rho, per-CTA APS sums (Eq. ebs, Eq. wafit)
         for (int p = 0; p < B; ++p) {
@@ -456,208 +469,236 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 continue;
             const ProblemDesc &pd = P.prob[p];
             const bool normalize = (pd.flags & RF_NORMALIZE) != 0;
-            if (w == 0) {  // the centre particle's total, by the same code as every particle's below
-                double S0;
-                int n0;
-                warp_particle_total(pd.part_S, pd.part_n, st[p].n_chunks, 0, lane, S0, n0);
-                if (lane == 0) {
-                    const float rho0 = fitness_rho(S0, st[p].nO, pd.tau, normalize);
-                    const bool centre = k == 1 || (pd.flags & RF_RHO_REF_CENTER) || pd.n_levels > 1;
-                    st[p].rho_ref = centre ? rho0 : st[p].rho_carry;
+            // A warp's lanes are 32 neighbouring particles and its chunks every FIT_WARPS-th,
+            // so every load of a partial is a contiguous run; the warps' sums meet in shared
+            // memory in a fixed order.  CTA b takes particles 32 b .. 32 b + 31, 32 (b + G) ..
+            // Bound by the FP64 additions (one a partial).  A warp per particle with its lanes
+            // over the chunks needs as many again for the butterfly: 37 us an iteration at
+            // 20,000 particles x 94 chunks against 13, 15 against 6 at 1024 x 110.
+            const int n_lvl = st[p].n_lvl, n_chunks = st[p].n_chunks;
+            auto share = [&](int i) {
+                double S = 0.0;
+                int nv = 0;
+                if (i < n_lvl) {
+#pragma unroll 8
+                    for (int ch = w; ch < n_chunks; ch += FIT_WARPS) {
+                        S += __ldcg(&pd.part_S[(size_t)ch * n_lvl + i]);
+                        nv += __ldcg(&pd.part_n[(size_t)ch * n_lvl + i]);
+                    }
                 }
+                share_S[w][lane] = S;
+                share_n[w][lane] = nv;
+            };
+            auto total = [&](int l, double &S, int &nv) {
+                S = share_S[0][l];
+                nv = share_n[0][l];
+#pragma unroll
+                for (int q = 1; q < FIT_WARPS; ++q) {
+                    S += share_S[q][l];
+                    nv += share_n[q][l];
+                }
+            };
+            const bool centre = k == 1 || (pd.flags & RF_RHO_REF_CENTER) || pd.n_levels > 1;
+            if (centre) {  // the centre particle's total, by the same sums as every particle's below
+                share(lane == 0 ? 0 : n_lvl);
+                __syncthreads();
+            }
+            if (tid == 0) {
+                double S0 = 0.0;
+                int n0;
+                if (centre)
+                    total(0, S0, n0);
+                st[p].rho_ref = centre ? fitness_rho(S0, st[p].nO, pd.tau, normalize) : st[p].rho_carry;
             }
             __syncthreads();
+            if (b * 32 >= n_lvl)
+                continue;  // no particles of this sequence for the CTA
             const float rho_ref = st[p].rho_ref;
             // particle 0 is the centre s*_{k-1} itself: an APS candidate only with RF_APS_WITH_CENTRE
             const int first = (pd.flags & RF_APS_WITH_CENTRE) ? 0 : 1;
             double sw = 0.0, swr = 0.0, swd[6] = {0, 0, 0, 0, 0, 0};
             int naps = 0, amax = -1;
-            long long valid = 0;  // valid TSDF samples of all particles (first corner case of Sec. 4)
+            int valid = 0;  // whether any particle has a valid TSDF sample (first corner case of Sec. 4)
             float rmax = -1.f, r2 = -1.f;
-            // one warp per particle: its lanes sum the chunk partials, lane 0 takes the particle
-            for (int i = b * FIT_WARPS + w; i < st[p].n_lvl; i += G * FIT_WARPS) {
-                double S;
-                int nv;
-                warp_particle_total(pd.part_S, pd.part_n, st[p].n_chunks, i, lane, S, nv);
-                if (lane != 0)
-                    continue;
-                valid += nv;
-                const float rho = fitness_rho(S, st[p].nO, pd.tau, normalize);
-                merge_max(rmax, amax, r2, rho, i, -1.f);
-                if (i >= first && rho > rho_ref) {
-                    const double wgt = (double)(rho - rho_ref);
-                    ++naps;
-                    sw += wgt;
-                    swr += wgt * (double)rho;
+            for (int i0 = b * 32; i0 < n_lvl; i0 += G * 32) {
+                share(i0 + lane);
+                __syncthreads();
+                const int i = i0 + lane;
+                if (w == 0 && i < n_lvl) {
+                    double S;
+                    int nv;
+                    total(lane, S, nv);
+                    valid |= nv != 0;
+                    const float rho = fitness_rho(S, st[p].nO, pd.tau, normalize);
+                    merge_max(rmax, amax, r2, rho, i, -1.f);
+                    if (i >= first && rho > rho_ref) {
+                        const double wgt = (double)(rho - rho_ref);
+                        ++naps;
+                        sw += wgt;
+                        swr += wgt * (double)rho;
 #pragma unroll
-                    for (int d = 0; d < 6; ++d)
-                        swd[d] += wgt * (double)(st[p].r[d] * __ldg(&pd.pst[(size_t)d * pd.n_tmpl + i]));
+                        for (int d = 0; d < 6; ++d)
+                            swd[d] += wgt * (double)(st[p].r[d] * __ldg(&pd.pst[(size_t)d * pd.n_tmpl + i]));
+                    }
                 }
+                __syncthreads();
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                sw += __shfl_xor_sync(0xffffffffu, sw, o);
-                swr += __shfl_xor_sync(0xffffffffu, swr, o);
-#pragma unroll
-                for (int d = 0; d < 6; ++d)
-                    swd[d] += __shfl_xor_sync(0xffffffffu, swd[d], o);
-                naps += __shfl_xor_sync(0xffffffffu, naps, o);
-                valid += __shfl_xor_sync(0xffffffffu, valid, o);
-                const float om = __shfl_xor_sync(0xffffffffu, rmax, o);
-                const int oa = __shfl_xor_sync(0xffffffffu, amax, o);
-                const float o2 = __shfl_xor_sync(0xffffffffu, r2, o);
-                merge_max(rmax, amax, r2, om, oa, o2);
-            }
-            if (lane == 0) {
-                red_d[w][0] = sw;
-                red_d[w][1] = swr;
-                for (int d = 0; d < 6; ++d)
-                    red_d[w][2 + d] = swd[d];
-                red_i[w][0] = naps;
-                red_i[w][1] = amax;
-                red_f[w][0] = rmax;
-                red_f[w][1] = r2;
-                red_v[w] = valid;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                int na = 0, am = -1;
-                long long nv_all = 0;
-                float rm = -1.f, rs = -1.f;
-                for (int q = 0; q < FIT_WARPS; ++q) {
-                    for (int e = 0; e < 8; ++e)
-                        acc[e] += red_d[q][e];
-                    na += red_i[q][0];
-                    nv_all += red_v[q];
-                    merge_max(rm, am, rs, red_f[q][0], red_i[q][1], red_f[q][1]);
+            if (w == 0) {  // the CTA's sums
+                double acc[8] = {sw, swr, swd[0], swd[1], swd[2], swd[3], swd[4], swd[5]};
+                const double mine = warp_sum8(acc, lane);
+                valid = __any_sync(0xffffffffu, valid);
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float om = __shfl_xor_sync(0xffffffffu, rmax, o);
+                    const int oa = __shfl_xor_sync(0xffffffffu, amax, o);
+                    const float o2 = __shfl_xor_sync(0xffffffffu, r2, o);
+                    merge_max(rmax, amax, r2, om, oa, o2);
                 }
+                naps = __reduce_add_sync(0xffffffffu, naps);
                 double *out = P.aps + ((size_t)b * MAX_BATCH + p) * APW;
-                for (int e = 0; e < 8; ++e)
-                    out[e] = acc[e];
-                out[8] = (double)na;
-                out[9] = (double)rm;
-                out[10] = (double)am;
-                out[11] = (double)rs;
-                out[12] = (double)nv_all;  // exact: far below 2^53
+                if (lane < 8)
+                    out[lane] = mine;
+                if (lane == 8)  // |APS| with a sign bit for "some valid sample", max, argmax, second
+                    *reinterpret_cast<int4 *>(out + 8) = make_int4(naps | (valid ? (int)0x80000000 : 0), __float_as_int(rmax),
+                                                                   amax, __float_as_int(r2));
             }
-            __syncthreads();
         }
-        if (!grid_barrier(P))
+        if (!grid_barrier(P, n_barriers))
             return;
-        // ---- phase C: fixed-order reduction of the APS sums and the PST update
-        for (int p = w; p < B; p += FIT_WARPS) {
+        // ---- phase C: fixed-order reduction of the APS sums and the PST update, the same in
+        // every CTA.  Warp e sums the CTAs' partials of quantity e (15 FP64 additions a warp;
+        // an FP64 instruction holds the SM's unit for 16 clocks, and both its CTAs do this);
+        // the last warp also merges the maxima and counts.  Then warp 0 updates the sequence
+        // with one axis per lane, so that the FP64 divisions of the six axes run side by side
+        // instead of one after another.  (One warp for everything took 17 to 20 us an
+        // iteration; this takes 5 at 1024 particles, 10 at 20,000.)
+        for (int p = 0; p < B; ++p) {
             if (!st[p].active)
                 continue;
-            const ProblemDesc &pd = P.prob[p];
-            PState &s = st[p];
-            double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            double na = 0.0, nvalid = 0.0;
-            float rm = -1.f, rs = -1.f;
-            int am = -1;
-            for (int q = lane; q < G; q += 32) {
-                const double *in = P.aps + ((size_t)q * MAX_BATCH + p) * APW;
-                for (int e = 0; e < 8; ++e)
-                    acc[e] += __ldcg(&in[e]);
-                na += __ldcg(&in[8]);
-                nvalid += __ldcg(&in[12]);
-                merge_max(rm, am, rs, (float)__ldcg(&in[9]), (int)__ldcg(&in[10]), (float)__ldcg(&in[11]));
+            const int parts = min(G, (st[p].n_lvl + 31) / 32);  // CTAs that had particles
+            {
+                double acc = 0.0;
+                for (int q = lane; q < parts; q += 32)
+                    acc += __ldcg(&P.aps[((size_t)q * MAX_BATCH + p) * APW + w]);
+                for (int o = 16; o > 0; o >>= 1)
+                    acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0)
+                    red_d[w] = acc;
+                if (w == FIT_WARPS - 1) {
+                    int na = 0, am = -1, any = 0;
+                    float rm = -1.f, rs = -1.f;
+                    for (int q = lane; q < parts; q += 32) {
+                        const int4 v = __ldcg(reinterpret_cast<const int4 *>(P.aps + ((size_t)q * MAX_BATCH + p) * APW + 8));
+                        na += v.x & 0x7FFFFFFF;
+                        any |= v.x < 0;
+                        merge_max(rm, am, rs, __int_as_float(v.y), v.z, __int_as_float(v.w));
+                    }
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const float om = __shfl_xor_sync(0xffffffffu, rm, o);
+                        const int oa = __shfl_xor_sync(0xffffffffu, am, o);
+                        const float o2 = __shfl_xor_sync(0xffffffffu, rs, o);
+                        merge_max(rm, am, rs, om, oa, o2);
+                    }
+                    na = __reduce_add_sync(0xffffffffu, na);
+                    any = __any_sync(0xffffffffu, any);
+                    if (lane == 0) {
+                        red_f[0] = rm;
+                        red_f[1] = rs;
+                        red_i[0] = am;
+                        red_i[1] = na;
+                        red_i[2] = any;
+                    }
+                }
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                for (int e = 0; e < 8; ++e)
-                    acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
-                na += __shfl_xor_sync(0xffffffffu, na, o);
-                nvalid += __shfl_xor_sync(0xffffffffu, nvalid, o);
-                const float om = __shfl_xor_sync(0xffffffffu, rm, o);
-                const int oa = __shfl_xor_sync(0xffffffffu, am, o);
-                const float o2 = __shfl_xor_sync(0xffffffffu, rs, o);
-                merge_max(rm, am, rs, om, oa, o2);
-            }
-            if (lane == 0) {
+            __syncthreads();
+            if (w == 0) {
+                const double v = lane < 8 ? red_d[lane] : 0.0;
+                const float rm = red_f[0], rs = red_f[1];
+                const int am = red_i[0], na = red_i[1];
+                const ProblemDesc &pd = P.prob[p];
+                PState &s = st[p];
                 // first corner case of Sec. 4: no particle found a single TSDF sample, so the
                 // likelihood cannot be evaluated: rho = 0.5, v = 1, r_hat = 0.5 v + eps, s* kept
-                const int corner = nvalid == 0.0 ? 1 : (na == 0.0 ? 2 : 0);
-                const int n_aps = corner == 1 ? 0 : (int)na;
+                const int corner = red_i[2] == 0 ? 1 : (na == 0 ? 2 : 0);
+                const int n_aps = corner == 1 ? 0 : na;
                 const float rho_ref = s.rho_ref;
-                float dbar[6], rhat[6];
-                float rho_t;
-                Pose s_new;
-                if (corner == 1) {
-                    rho_t = 0.5f;
-                    for (int d = 0; d < 6; ++d) {
-                        dbar[d] = 0.f;
-                        rhat[d] = (float)(0.5 + (double)pd.eps);
-                    }
-                    s_new = s.c;
-                    s.empty_run += 1;
-                } else if (n_aps > 0) {
-                    double nv2 = 0.0, db[6];
-                    for (int d = 0; d < 6; ++d) {
-                        db[d] = acc[2 + d] / acc[0];
-                        nv2 += db[d] * db[d];
-                    }
-                    const double nv = sqrt(nv2);
-                    rho_t = (float)(acc[1] / acc[0]);
-                    for (int d = 0; d < 6; ++d) {
-                        dbar[d] = (float)db[d];
-                        const double dir = nv < 1e-12 ? 0.40824829046386302 : fabs(db[d]) / nv;
-                        rhat[d] = (float)((1.0 - (double)rho_t) * dir + (double)pd.eps);
-                    }
-                    compose_offset(s.c, dbar, (pd.flags & RF_RIGHT_MULT) != 0, s_new);
-                    s.empty_run = 0;
-                } else {
-                    rho_t = rho_ref;
-                    for (int d = 0; d < 6; ++d) {
-                        dbar[d] = 0.f;
-                        rhat[d] = (float)(2.0 * (1.0 - (double)rho_ref) * 0.40824829046386302 + (double)pd.eps);
-                    }
-                    s_new = s.c;
-                    s.empty_run += 1;
+                // lane 1: Eq. wafit; lanes 2 .. 7: the offsets of Eq. ebs, axis d on lane 2 + d
+                const double sw = __shfl_sync(0xffffffffu, v, 0);
+                const double quo = n_aps > 0 ? v / sw : 0.0;
+                const float rho_t = corner == 1 ? 0.5f : (n_aps > 0 ? (float)__shfl_sync(0xffffffffu, quo, 1) : rho_ref);
+                float dbar[6];
+                double nv2 = 0.0;
+#pragma unroll
+                for (int d = 0; d < 6; ++d) {
+                    const double db = __shfl_sync(0xffffffffu, quo, 2 + d);
+                    dbar[d] = (float)db;
+                    nv2 += db * db;
                 }
-                for (int d = 0; d < 6; ++d)
-                    s.r[d] = pd.beta * s.r[d] + (1.f - pd.beta) * rhat[d];
-                s.rho_carry = rho_t;
-                s.c = s_new;
-                if (k == 1)
-                    for (int d = 0; d < 6; ++d)
+                const double nv = sqrt(nv2);
+                float rhat;
+                if (corner == 1) {
+                    rhat = (float)(0.5 + (double)pd.eps);
+                } else if (n_aps > 0) {
+                    const double dir = nv < 1e-12 ? 0.40824829046386302 : fabs(quo) / nv;
+                    rhat = (float)((1.0 - (double)rho_t) * dir + (double)pd.eps);
+                } else {
+                    rhat = (float)(2.0 * (1.0 - (double)rho_ref) * 0.40824829046386302 + (double)pd.eps);
+                }
+                if (lane >= 2 && lane < 8) {
+                    const int d = lane - 2;
+                    s.r[d] = pd.beta * s.r[d] + (1.f - pd.beta) * rhat;
+                    if (k == 1)
                         s.r1[d] = s.r[d];
-                float step = 0.f;
-                for (int d = 0; d < 6; ++d)
-                    step = fmaxf(step, fabsf(dbar[d]));
-                int stop = 0;
-                if (s.empty_run >= 2)
-                    stop = 1;
-                else if (n_aps > 0 && step < pd.stop_eps)
-                    stop = 2;
-                else if (k == pd.k_max)
-                    stop = 3;
-                s.stop = stop;
-                s.lookups += (long long)s.nO * (long long)s.n_lvl;
-                if (b == 0 && pd.stats) {
-                    rf_iter_stats &row = pd.stats->it[k - 1];
-                    row.k = k;
-                    row.n_overlap = s.nO;
-                    row.n_aps = n_aps;
-                    row.argmax = am;
-                    row.rho_ref = rho_ref;
-                    row.rho_tilde = rho_t;
-                    row.rho_max = rm;
-                    row.rho_second = rs;
-                    for (int a = 0; a < 4; ++a)
-                        row.pose[a] = s.c.q[a];
-                    for (int a = 0; a < 3; ++a)
-                        row.pose[4 + a] = s.c.t[a];
-                    for (int d = 0; d < 6; ++d) {
-                        row.scale[d] = s.r[d];
-                        row.offset[d] = dbar[d];
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    if (n_aps > 0) {
+                        Pose s_new;
+                        compose_offset(s.c, dbar, (pd.flags & RF_RIGHT_MULT) != 0, s_new);
+                        s.c = s_new;
+                        s.empty_run = 0;
+                    } else {
+                        s.empty_run += 1;
                     }
-                    row.stop = stop;
-                    row.level = s.level;
-                    row.n_particles = s.n_lvl;
-                    row.corner = corner;
+                    s.rho_carry = rho_t;
+                    float step = 0.f;
+                    for (int d = 0; d < 6; ++d)
+                        step = fmaxf(step, fabsf(dbar[d]));
+                    int stop = 0;
+                    if (s.empty_run >= 2)
+                        stop = 1;
+                    else if (n_aps > 0 && step < pd.stop_eps)
+                        stop = 2;
+                    else if (k == pd.k_max)
+                        stop = 3;
+                    s.stop = stop;
+                    s.lookups += (long long)s.nO * (long long)s.n_lvl;
+                    if (b == 0 && pd.stats) {
+                        rf_iter_stats &row = pd.stats->it[k - 1];
+                        row.k = k;
+                        row.n_overlap = s.nO;
+                        row.n_aps = n_aps;
+                        row.argmax = am;
+                        row.rho_ref = rho_ref;
+                        row.rho_tilde = rho_t;
+                        row.rho_max = rm;
+                        row.rho_second = rs;
+                        for (int a = 0; a < 4; ++a)
+                            row.pose[a] = s.c.q[a];
+                        for (int a = 0; a < 3; ++a)
+                            row.pose[4 + a] = s.c.t[a];
+                        for (int d = 0; d < 6; ++d) {
+                            row.scale[d] = s.r[d];
+                            row.offset[d] = dbar[d];
+                        }
+                        row.stop = stop;
+                        row.level = s.level;
+                        row.n_particles = s.n_lvl;
+                        row.corner = corner;
+                    }
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
     }
     // ---- epilogue (CTA 0): final poses, r_1 for the next frame, summaries
     if (b == 0 && tid < B && st[tid].stop != 5) {
