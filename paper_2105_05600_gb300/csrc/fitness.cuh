@@ -15,8 +15,10 @@ Pose to_pose(const rf_pose &p);
 
 constexpr int FIT_THREADS = 256;
 constexpr int FIT_WARPS = FIT_THREADS / 32;
-constexpr int CHUNK_MAX = 256;        // points staged per warp (16 B each)
+constexpr int GROUP_PARTICLES = 64;   // particles of a warp's work unit, two per lane
+constexpr int CHUNK_MAX = 256;        // points staged at once
 constexpr int MIN_CHUNK = 32;         // fewest points per work unit
+constexpr int SMALL_CHUNK = 24;       // fewest where there are not enough units for the warps
 #ifndef RF_UNITS_PER_WARP
 #define RF_UNITS_PER_WARP 16
 #endif
@@ -24,15 +26,14 @@ constexpr int UNITS_PER_WARP = RF_UNITS_PER_WARP;  // target work units per warp
 constexpr int APW = 16;               // doubles per CTA in the APS partials: 8 sums, then one int4
 constexpr int MAX_CTAS_PER_SM = 2048 / FIT_THREADS;  // bound for grid-sized scratch
 // CTAs of the persistent kernel resident per SM (register budget 65536 / (256 * n)).
-// Measured on the paper-scale frame: groups of 6 lookups at 2 CTAs per SM 312.7 G
-// lookups/s, 8 at 2: 306.5, 4 at 3: 299.1 (more loads in flight per warp beat
-// more warps).
+// 3 leave 80 registers for the pair loop, which spills: 15.7 ms against 13.9 ms for a
+// paper-scale frame.
 #ifndef RF_PFO_MIN_BLOCKS
 #define RF_PFO_MIN_BLOCKS 2
 #endif
-// lookups whose loads are issued together in the trilinear loop (the default;
-// the persistent kernel is also built for groups of 4 and 8, picked by the
-// launch configuration)
+// Points whose terms are added before the compensated sum, half of them (for two
+// particles each: GROUP lookups) with their loads in flight together; the default.
+// The persistent kernel is also built for 4 and 8, picked by the launch configuration.
 #ifndef RF_GROUP
 #define RF_GROUP 6
 #endif
@@ -105,250 +106,247 @@ struct FitParams {
     int l1, right_mult;
 };
 
-template <int DT, int MODE, bool L1, int G>
-__device__ __forceinline__ void fitness_points(const CellView &V, const float4 *spts, int cnt, const float R[9],
-                                               float t0, float t1, float t2, float &sum, float &comp, int &nv);
-
-// Lane `lane` of a warp scores particle i over the points staged in `spts`
-// [0, cnt): S = sum psi^2 (|psi| with L1), psi = 1 for invalid samples; G
-// lookups have their loads in flight together.
-template <int DT, int MODE, int G = GROUP>
-__device__ __forceinline__ void fitness_lane(const VolumeDesc &V, const float4 *spts, int cnt, const FitParams &fp,
-                                             int i, double &S_out, int &n_out)
+// Pose of particle i (centre (+) (scale . omega_i)), folded with the world ->
+// voxel-centre map g = p / voxel - origin / voxel - 1/2, so that a point goes
+// straight to grid units.
+__device__ __forceinline__ void particle_pose(const VolumeDesc &V, const FitParams &fp, int i, float R[9], float t[3])
 {
     Pose P;
-    {
-        const int ii = i < fp.n ? i : 0;
-        float d[6];
+    float d[6];
 #pragma unroll
-        for (int a = 0; a < 6; ++a)
-            d[a] = fp.r[a] * __ldg(&fp.pst[(size_t)a * fp.ld + ii]);
-        compose_offset(fp.c, d, fp.right_mult != 0, P);
-    }
-    // the rotation and translation are folded with the world -> voxel-centre map
-    // g = p / voxel - origin / voxel - 1/2, so a point goes straight to grid units
-    float R[9];
+    for (int a = 0; a < 6; ++a)
+        d[a] = fp.r[a] * __ldg(&fp.pst[(size_t)a * fp.ld + i]);
+    compose_offset(fp.c, d, fp.right_mult != 0, P);
     quat_rot(P.q, R);
     const float s = V.inv_voxel;
+#pragma unroll
     for (int a = 0; a < 9; ++a)
         R[a] *= s;
-    const float t0 = fmaf(P.t[0], s, V.goff[0]), t1 = fmaf(P.t[1], s, V.goff[1]), t2 = fmaf(P.t[2], s, V.goff[2]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        t[a] = fmaf(P.t[a], s, V.goff[a]);
+}
+
+// Points of a unit staged for the pair loop: every coordinate twice, so that one
+// 16-byte and one 8-byte broadcast load give the (x, x), (y, y), (z, z) operands.
+struct PairPoints {
+    ulonglong2 xy[CHUNK_MAX];
+    f2_t z[CHUNK_MAX];
+};
+
+// Grid-space poses of a lane's two particles, component by component.
+struct PairPose {
+    f2_t R[9], t[3];
+};
+
+// psi of points j .. j + N - 1 for both particles of a lane.  What bounds it on a
+// GB300: the FP32 pipe (a .f32x2 instruction holds it two clocks, so pairs save issue
+// slots, not arithmetic: 56 instructions a lookup against 80 for the scalar loop of one
+// particle per lane, 61 of 124 clocks a scheduler in use) and, for wide swarms, the
+// lines a warp's loads touch (one a clock).  All class bytes are loaded, then all
+// records, then used.  Three ways through, by warp vote, since a
+// wide swarm spends most of its lookups in constant bricks and a converged one
+// none: every lookup constant (no record, psi = 1), every lookup mixed (plain
+// loads), or both (loads predicated on the class).  321 M lookups of a converged / a
+// mixed / a wide swarm (int16, 20,000 particles, sorted) take 0.77 / 0.83 / 0.91 ms
+// against 1.08 / 1.19 / 1.18 ms for the scalar loop.  `live` of the points count as
+// lookups (the rest repeat the last one).
+template <int DT, int N>
+__device__ __forceinline__ void pair_lookups(const CellView &V, const PairPoints &sp, int j, int last, int live,
+                                             const PairPose &P, f2_t psi[N], int &nva, int &nvb)
+{
+    const f2_t MAGIC = f2_pack(FLOOR_MAGIC, FLOOR_MAGIC);
+    f2_t FX[N], FY[N], FZ[N];
+    unsigned ra[N], rb[N];
+    int ca[N], cb[N], any = 0, all = -1;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const int q = min(j + u, last);
+        const ulonglong2 xy = sp.xy[q];
+        const f2_t X = xy.x, Y = xy.y, Z = sp.z[q];
+        const f2_t GX = f2_fma(P.R[0], X, f2_fma(P.R[1], Y, f2_fma(P.R[2], Z, P.t[0])));
+        const f2_t GY = f2_fma(P.R[3], X, f2_fma(P.R[4], Y, f2_fma(P.R[5], Z, P.t[1])));
+        const f2_t GZ = f2_fma(P.R[6], X, f2_fma(P.R[7], Y, f2_fma(P.R[8], Z, P.t[2])));
+        const f2_t TX = f2_add_rd(GX, MAGIC), TY = f2_add_rd(GY, MAGIC), TZ = f2_add_rd(GZ, MAGIC);
+        FX[u] = f2_sub(GX, f2_sub(TX, MAGIC));
+        FY[u] = f2_sub(GY, f2_sub(TY, MAGIC));
+        FZ[u] = f2_sub(GZ, f2_sub(TZ, MAGIC));
+        float xa, xb, ya, yb, za, zb;
+        f2_unpack(TX, xa, xb);
+        f2_unpack(TY, ya, yb);
+        f2_unpack(TZ, za, zb);
+        ra[u] = cell_record(V, xa, ya, za);
+        rb[u] = cell_record(V, xb, yb, zb);
+        ca[u] = __ldg(V.cls + (ra[u] >> 9));
+        cb[u] = __ldg(V.cls + (rb[u] >> 9));
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        any |= ca[u] | cb[u];
+        all &= ca[u] & cb[u];
+    }
+    if (__any_sync(0xffffffffu, any < 0)) {
+        CellData<DT> da[N], db[N];
+        if (__all_sync(0xffffffffu, all < 0)) {
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                cell_fetch<DT, false>(V, ra[u], 0, da[u]);
+                cell_fetch<DT, false>(V, rb[u], 0, db[u]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                cell_fetch<DT, true>(V, ra[u], ca[u], da[u]);
+                cell_fetch<DT, true>(V, rb[u], cb[u], db[u]);
+                nva += u < live ? max(ca[u], 0) : 0;  // free space is valid
+                nvb += u < live ? max(cb[u], 0) : 0;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            bool oka, okb;
+            psi[u] = cell_eval<DT>(FX[u], FY[u], FZ[u], da[u], db[u], oka, okb);
+            nva += (oka && u < live) ? 1 : 0;
+            nvb += (okb && u < live) ? 1 : 0;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            psi[u] = 0x3F8000003F800000ull;
+            nva += u < live ? ca[u] : 0;
+            nvb += u < live ? cb[u] : 0;
+        }
+    }
+}
+
+// One lane scores particles ia and ib over the staged points [0, cnt):
+// S = sum psi^2 (|psi| with L1), psi = 1 for invalid samples.  Both particles go
+// through the same operations side by side, so a particle's sum does not depend
+// on its partner.  G terms are added plainly (a partial of <= G terms in [0, 1]),
+// then joined to the total with compensation.
+template <int DT, int MODE, int G, bool L1>
+__device__ __forceinline__ void fitness_pair(const VolumeDesc &Vd, const PairPoints &sp, int cnt, const FitParams &fp,
+                                             int ia, int ib, double S_out[2], int n_out[2])
+{
+    // points in flight at once (a float record takes 8 registers: 3 in flight spill,
+    // 454 against 398 us for 9973 particles x 8.4 k points)
+    constexpr int N = DT == RF_F32 ? 2 : G / 2;
+    static_assert(G % N == 0, "whole batches per group");
+    PairPose P;
+    {
+        float R[2][9], t[2][3];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            particle_pose(Vd, fp, h ? ib : ia, R[h], t[h]);
+#pragma unroll
+        for (int a = 0; a < 9; ++a)
+            P.R[a] = f2_pack(R[0][a], R[1][a]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            P.t[a] = f2_pack(t[0][a], t[1][a]);
+    }
+    const CellView V(Vd);
+    float sum[2] = {0.f, 0.f}, comp[2] = {0.f, 0.f};
+    int nv[2] = {0, 0};
+    auto add = [&](float a, float b) {
+        if (Mode<MODE>::plain) {
+            sum[0] += a;
+            sum[1] += b;
+        } else {
+            neumaier_add(sum[0], comp[0], a);
+            neumaier_add(sum[1], comp[1], b);
+        }
+    };
+    int j = 0;
+    for (; j + G <= cnt; j += G) {
+        f2_t grp = 0ull;
+#pragma unroll
+        for (int h = 0; h < G; h += N) {
+            f2_t psi[N];
+            pair_lookups<DT, N>(V, sp, j + h, cnt - 1, N, P, psi, nv[0], nv[1]);
+#pragma unroll
+            for (int u = 0; u < N; ++u)
+                grp = L1 ? f2_add(grp, psi[u] & 0x7FFFFFFF7FFFFFFFull) : f2_fma(psi[u], psi[u], grp);
+        }
+        float a, b;
+        f2_unpack(grp, a, b);
+        add(a, b);
+    }
+    for (; j < cnt; j += N) {  // the tail: term by term
+        f2_t psi[N];
+        pair_lookups<DT, N>(V, sp, j, cnt - 1, cnt - j, P, psi, nv[0], nv[1]);
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (j + u < cnt) {
+                float a, b;
+                f2_unpack(L1 ? psi[u] & 0x7FFFFFFF7FFFFFFFull : f2_mul(psi[u], psi[u]), a, b);
+                add(a, b);
+            }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        S_out[h] = (double)sum[h] + (double)comp[h];
+        n_out[h] = nv[h];
+    }
+}
+
+// Nearest-voxel lookups of one particle over the staged points.
+template <int DT, int MODE>
+__device__ __forceinline__ void fitness_nearest(const VolumeDesc &Vd, const PairPoints &sp, int cnt, const FitParams &fp,
+                                                int i, double &S_out, int &n_out)
+{
+    float R[9], t[3];
+    particle_pose(Vd, fp, i, R, t);
+    const CellView V(Vd);
     float sum = 0.f, comp = 0.f;
     int nv = 0;
-    const CellView cv(V);
-    if (fp.l1)
-        fitness_points<DT, MODE, true, G>(cv, spts, cnt, R, t0, t1, t2, sum, comp, nv);
-    else
-        fitness_points<DT, MODE, false, G>(cv, spts, cnt, R, t0, t1, t2, sum, comp, nv);
+    for (int j = 0; j < cnt; ++j) {
+        const ulonglong2 xy = sp.xy[j];
+        const float x = __uint_as_float((unsigned)xy.x), y = __uint_as_float((unsigned)xy.y),
+                    z = __uint_as_float((unsigned)sp.z[j]);
+        float psi;
+        const bool ok = sample_nearest_g<DT>(V, fmaf(R[0], x, fmaf(R[1], y, fmaf(R[2], z, t[0]))),
+                                             fmaf(R[3], x, fmaf(R[4], y, fmaf(R[5], z, t[1]))),
+                                             fmaf(R[6], x, fmaf(R[7], y, fmaf(R[8], z, t[2]))), psi);
+        nv += ok ? 1 : 0;
+        psi = ok ? psi : 1.f;
+        const float term = fp.l1 ? fabsf(psi) : psi * psi;
+        if (Mode<MODE>::plain)
+            sum += term;
+        else
+            neumaier_add(sum, comp, term);
+    }
     S_out = (double)sum + (double)comp;
     n_out = nv;
 }
 
-// ------------------------------------------------------------------ packed FP32 pairs
-// Blackwell's FP32 pair instructions (fma/add/sub/mul .f32x2): two independent
-// IEEE operations per instruction, each rounded exactly as its scalar form.  The
-// packed int16 loop below pairs two points of a group and performs, for each of
-// them, the same operations in the same order as the scalar loop, so its results
-// are bit-identical with fewer issued instructions.
-#ifndef RF_PACKED
-#define RF_PACKED 0
-#endif
-typedef unsigned long long f2_t;
-__device__ __forceinline__ f2_t f2_pack(float a, float b)
+// Point j of a unit, staged.
+__device__ __forceinline__ void stage_point(PairPoints &sp, int j, const float4 &p)
 {
-    f2_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2_t r, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c)
-{
-    f2_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2_t f2_add_rd(f2_t a, f2_t b)
-{
-    f2_t d;
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2_t f2_sub(f2_t a, f2_t b)
-{
-    f2_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b)
-{
-    f2_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
+    sp.xy[j] = make_ulonglong2(f2_pack(p.x, p.x), f2_pack(p.y, p.y));
+    sp.z[j] = f2_pack(p.z, p.z);
 }
 
-// cell_locate from the biased floor words (bits of __fadd_rd(g, 1.5 * 2^23)).
-__device__ __forceinline__ void cell_locate_int(const CellView &V, int ix, int iy, int iz, unsigned &rec, unsigned &cls)
+// A warp's share of a work unit: 64 particles (two per lane) over the staged points.  Particles beyond the swarm repeat the first one.
+template <int DT, int MODE, int G = GROUP>
+__device__ __forceinline__ void fitness_unit(const VolumeDesc &V, const PairPoints &sp, int cnt, const FitParams &fp,
+                                             const int i[2], double S[2], int nv[2])
 {
-    const bool inside = (unsigned)ix < (unsigned)(V.dim[0] - 1) && (unsigned)iy < (unsigned)(V.dim[1] - 1) &&
-                        (unsigned)iz < (unsigned)(V.dim[2] - 1);
-    const unsigned brick =
-        (unsigned)(ix >> 3) + (unsigned)V.nb0 * ((unsigned)(iy >> 3) + (unsigned)V.nb1 * (unsigned)(iz >> 3));
-    rec = brick * (unsigned)BRICK_VOX + (unsigned)((ix & 7) | ((iy & 7) << 3) | ((iz & 7) << 6));
-    cls = inside ? (unsigned)__ldg(&V.cls[brick]) : (unsigned)CELLS_INVALID;
-}
-
-// The int16 trilinear group loop with two points per packed instruction (G even).
-// Per point: the transform, floor and fraction, the class and record loads, the
-// decode and the interpolation of the scalar loop, operation for operation.
-template <int MODE, bool L1, int G>
-__device__ __forceinline__ int fitness_points_i16_packed(const CellView &V, const float4 *spts, int cnt,
-                                                         const float R[9], float t0, float t1, float t2, float &sum,
-                                                         float &comp, int &nv)
-{
-    static_assert(G % 2 == 0, "the packed loop pairs the points of a group");
-    const f2_t R0 = f2_pack(R[0], R[0]), R1 = f2_pack(R[1], R[1]), R2 = f2_pack(R[2], R[2]);
-    const f2_t R3 = f2_pack(R[3], R[3]), R4 = f2_pack(R[4], R[4]), R5 = f2_pack(R[5], R[5]);
-    const f2_t R6 = f2_pack(R[6], R[6]), R7 = f2_pack(R[7], R[7]), R8 = f2_pack(R[8], R[8]);
-    const f2_t T0 = f2_pack(t0, t0), T1 = f2_pack(t1, t1), T2 = f2_pack(t2, t2);
-    const f2_t MAGIC = f2_pack(12582912.0f, 12582912.0f);
-    const f2_t BIAS = f2_pack(8421376.0f, 8421376.0f);  // 2^23 + 32768
-    const f2_t SCALE = f2_pack(1.0f / I16_SCALE, 1.0f / I16_SCALE);
-    int j = 0;
-    for (; j + G <= cnt; j += G) {
-        f2_t FX[G / 2], FY[G / 2], FZ[G / 2];
-        CellRef c[G];
-        CellData<RF_I16> d[G];
-#pragma unroll
-        for (int p = 0; p < G / 2; ++p) {
-            const float4 xa = spts[j + 2 * p], xb = spts[j + 2 * p + 1];
-            const f2_t X = f2_pack(xa.x, xb.x), Y = f2_pack(xa.y, xb.y), Z = f2_pack(xa.z, xb.z);
-            const f2_t GX = f2_fma(R0, X, f2_fma(R1, Y, f2_fma(R2, Z, T0)));
-            const f2_t GY = f2_fma(R3, X, f2_fma(R4, Y, f2_fma(R5, Z, T1)));
-            const f2_t GZ = f2_fma(R6, X, f2_fma(R7, Y, f2_fma(R8, Z, T2)));
-            const f2_t TX = f2_add_rd(GX, MAGIC), TY = f2_add_rd(GY, MAGIC), TZ = f2_add_rd(GZ, MAGIC);
-            FX[p] = f2_sub(GX, f2_sub(TX, MAGIC));
-            FY[p] = f2_sub(GY, f2_sub(TY, MAGIC));
-            FZ[p] = f2_sub(GZ, f2_sub(TZ, MAGIC));
-            float txa, txb, tya, tyb, tza, tzb;
-            f2_unpack(TX, txa, txb);
-            f2_unpack(TY, tya, tyb);
-            f2_unpack(TZ, tza, tzb);
-            cell_locate_int(V, __float_as_int(txa) - 0x4B400000, __float_as_int(tya) - 0x4B400000,
-                            __float_as_int(tza) - 0x4B400000, c[2 * p].rec, c[2 * p].cls);
-            cell_locate_int(V, __float_as_int(txb) - 0x4B400000, __float_as_int(tyb) - 0x4B400000,
-                            __float_as_int(tzb) - 0x4B400000, c[2 * p + 1].rec, c[2 * p + 1].cls);
-        }
-#pragma unroll
-        for (int u = 0; u < G; ++u)
-            cell_fetch<RF_I16>(V, c[u], d[u]);
-        float grp = 0.f;
-#pragma unroll
-        for (int p = 0; p < G / 2; ++p) {
-            const uint4 a = d[2 * p].a, b = d[2 * p + 1].a;
-            // biased corner codes as exact floats 2^23 + u, the two points side by side
-            auto lo = [](uint32_t w) { return __int_as_float((int)__byte_perm(w, 0x4B00u, 0x5410)); };
-            auto hi = [](uint32_t w) { return __int_as_float((int)__byte_perm(w, 0x4B00u, 0x5432)); };
-            const f2_t A0 = f2_pack(lo(a.x), lo(b.x)), A1 = f2_pack(hi(a.x), hi(b.x));
-            const f2_t A2 = f2_pack(lo(a.y), lo(b.y)), A3 = f2_pack(hi(a.y), hi(b.y));
-            const f2_t A4 = f2_pack(lo(a.z), lo(b.z)), A5 = f2_pack(hi(a.z), hi(b.z));
-            const f2_t A6 = f2_pack(lo(a.w), lo(b.w)), A7 = f2_pack(hi(a.w), hi(b.w));
-            const f2_t C00 = f2_fma(FX[p], f2_sub(A1, A0), f2_sub(A0, BIAS));
-            const f2_t C10 = f2_fma(FX[p], f2_sub(A3, A2), f2_sub(A2, BIAS));
-            const f2_t C01 = f2_fma(FX[p], f2_sub(A5, A4), f2_sub(A4, BIAS));
-            const f2_t C11 = f2_fma(FX[p], f2_sub(A7, A6), f2_sub(A6, BIAS));
-            const f2_t Y0 = f2_fma(FY[p], f2_sub(C10, C00), C00);
-            const f2_t Y1 = f2_fma(FY[p], f2_sub(C11, C01), C01);
-            const f2_t VV = f2_mul(f2_fma(FZ[p], f2_sub(Y1, Y0), Y0), SCALE);
-            float va, vb;
-            f2_unpack(VV, va, vb);
-            const bool oka = (a.x & 0xFFFFu) != 0u, okb = (b.x & 0xFFFFu) != 0u;
-            nv += (oka ? 1 : 0) + (okb ? 1 : 0);
-            va = oka ? va : 1.f;
-            vb = okb ? vb : 1.f;
-            grp += L1 ? fabsf(va) : va * va;
-            grp += L1 ? fabsf(vb) : vb * vb;
-        }
-        if (Mode<MODE>::plain)
-            sum += grp;
-        else
-            neumaier_add(sum, comp, grp);
-    }
-    return j;
-}
-
-// The point loop of one lane: lookups of points [0, cnt) under the grid-space
-// pose (R, t), accumulated as psi^2 (|psi| with L1), psi = 1 when invalid.
-template <int DT, int MODE, bool L1, int G>
-__device__ __forceinline__ void fitness_points(const CellView &V, const float4 *spts, int cnt, const float R[9],
-                                               float t0, float t1, float t2, float &sum, float &comp, int &nv)
-{
-    int j = 0;
-    auto add = [&](float grp) {
-        if (Mode<MODE>::plain)
-            sum += grp;
-        else
-            neumaier_add(sum, comp, grp);
-    };
-    auto term = [&](bool ok, float psi) {  // psi = 1 when invalid (cell_eval, nearest below)
-        nv += ok ? 1 : 0;
-        return L1 ? fabsf(psi) : psi * psi;
-    };
-    if constexpr (RF_PACKED && DT == RF_I16 && !Mode<MODE>::nearest && G % 2 == 0)
-        j = fitness_points_i16_packed<MODE, L1, G>(V, spts, cnt, R, t0, t1, t2, sum, comp, nv);
-    else if (!Mode<MODE>::nearest) {
-        // groups of G lookups: all class loads, then all cell loads, then the
-        // arithmetic, so each group pays the load latency once; a plain FP32
-        // partial of <= G terms in [0, 1] is then added with compensation
-        for (; j + G <= cnt; j += G) {
-            CellRef c[G];
-            CellData<DT> d[G];
-#pragma unroll
-            for (int u = 0; u < G; ++u) {
-                const float4 x = spts[j + u];
-                cell_locate(V, fmaf(R[0], x.x, fmaf(R[1], x.y, fmaf(R[2], x.z, t0))),
-                            fmaf(R[3], x.x, fmaf(R[4], x.y, fmaf(R[5], x.z, t1))),
-                            fmaf(R[6], x.x, fmaf(R[7], x.y, fmaf(R[8], x.z, t2))), c[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < G; ++u)
-                cell_fetch<DT>(V, c[u], d[u]);
-            float grp = 0.f;
-#pragma unroll
-            for (int u = 0; u < G; ++u) {
-                float psi;
-                const bool ok = cell_eval<DT>(c[u], d[u], psi);
-                grp += term(ok, psi);
-            }
-            add(grp);
-        }
-    }
-    for (; j < cnt; ++j) {  // the tail of the chunk (or every point in nearest mode)
-        const float4 x = spts[j];
-        const float gx = fmaf(R[0], x.x, fmaf(R[1], x.y, fmaf(R[2], x.z, t0)));
-        const float gy = fmaf(R[3], x.x, fmaf(R[4], x.y, fmaf(R[5], x.z, t1)));
-        const float gz = fmaf(R[6], x.x, fmaf(R[7], x.y, fmaf(R[8], x.z, t2)));
-        float psi;
-        bool ok;
-        if (Mode<MODE>::nearest) {
-            ok = sample_nearest_g<DT>(V, gx, gy, gz, psi);
-            psi = ok ? psi : 1.f;
-        } else {
-            CellRef c;
-            CellData<DT> d;
-            cell_locate(V, gx, gy, gz, c);
-            cell_fetch<DT>(V, c, d);
-            ok = cell_eval<DT>(c, d, psi);
-        }
-        add(term(ok, psi));
+    const int ia = i[0] < fp.n ? i[0] : 0, ib = i[1] < fp.n ? i[1] : 0;
+    if constexpr (Mode<MODE>::nearest) {
+        fitness_nearest<DT, MODE>(V, sp, cnt, fp, ia, S[0], nv[0]);
+        fitness_nearest<DT, MODE>(V, sp, cnt, fp, ib, S[1], nv[1]);
+    } else if (fp.l1) {
+        fitness_pair<DT, MODE, G, true>(V, sp, cnt, fp, ia, ib, S, nv);
+    } else {
+        fitness_pair<DT, MODE, G, false>(V, sp, cnt, fp, ia, ib, S, nv);
     }
 }
 
-// Work decomposition shared by the standalone and the persistent kernels: unit
-// u = (point chunk u / groups, particle group u % groups); consecutive units
-// share a point chunk so the warps of a CTA touch neighbouring voxels.
+// Work decomposition shared by the standalone and the persistent kernels: (point
+// chunk, group of GROUP_PARTICLES particles, two per lane of a warp).  Consecutive
+// groups share a point chunk, so that neighbouring warps read the same part of the
+// volume.
 struct Split {
     int groups, n_chunks, chunk;
 };
@@ -356,20 +354,21 @@ struct Split {
 __host__ __device__ inline Split make_split(int n, int m, int total_warps, int max_chunks)
 {
     Split s;
-    s.groups = (n + 31) / 32;
-    int want = (UNITS_PER_WARP * total_warps + s.groups - 1) / s.groups;
+    s.groups = (n + GROUP_PARTICLES - 1) / GROUP_PARTICLES;
+    const int g32 = (n + 31) / 32;  // the chunk length is chosen for groups of 32 particles
+    int want = (UNITS_PER_WARP * total_warps + g32 - 1) / g32;
     int lo = (m + CHUNK_MAX - 1) / CHUNK_MAX;   // staging capacity
     int hi = (m + MIN_CHUNK - 1) / MIN_CHUNK;   // at least MIN_CHUNK points per unit
+    if (s.groups * hi < total_warps)  // (1024 particles x 4800 points: 582 -> 536 us a frame)
+        hi = (m + SMALL_CHUNK - 1) / SMALL_CHUNK;
     want = want < lo ? lo : want;
     want = want > hi ? hi : want;
     want = want > max_chunks ? max_chunks : want;
     want = want < 1 ? 1 : want;
-    s.n_chunks = want;
     s.chunk = (m + want - 1) / want;
-    if (s.chunk > CHUNK_MAX) {  // only when max_chunks binds
+    if (s.chunk > CHUNK_MAX)  // only when max_chunks binds
         s.chunk = CHUNK_MAX;
-        s.n_chunks = (m + CHUNK_MAX - 1) / CHUNK_MAX;
-    }
+    s.n_chunks = (m + s.chunk - 1) / s.chunk;  // every chunk holds a point
     return s;
 }
 
@@ -378,59 +377,7 @@ __host__ inline int max_chunks_for(int n, int m_max, int total_warps)
     const int groups = (n + 31) / 32;
     const int a = (UNITS_PER_WARP * total_warps + groups - 1) / groups;
     const int b = (m_max + CHUNK_MAX - 1) / CHUNK_MAX;
-    return std::max(1, std::max(std::min(a, (m_max + MIN_CHUNK - 1) / MIN_CHUNK), b));
-}
-
-// All warps of the grid walk the units; each stages its chunk of points, scores
-// its 32 particles and writes one (S, n) partial per particle.  `coherent`
-// selects L2-coherent loads for points written earlier in the same kernel.
-// With a unit counter (`next_unit` non-null, zero at the start of the phase) the
-// warps take units dynamically, one atomic per unit, fetched one unit ahead;
-// otherwise warp w takes units w, w + total_warps, ...
-template <int DT, int MODE, bool COHERENT>
-__device__ __forceinline__ void fitness_units(const VolumeDesc &V, const float4 *pts, int m, const FitParams &fp,
-                                              const Split &sp, double *part_S, int *part_n, float4 *smem_pts,
-                                              int warp_global, int total_warps, int lane, int warp_in_block,
-                                              int *next_unit = nullptr)
-{
-    float4 *spts = smem_pts + (size_t)warp_in_block * CHUNK_MAX;
-    const int units = sp.groups * sp.n_chunks;
-    int staged = -1;
-    int u = warp_global;
-    if (next_unit) {
-        int t = 0;
-        if (lane == 0)
-            t = atomicAdd(next_unit, 1);
-        u = __shfl_sync(0xffffffffu, t, 0);
-    }
-    while (u < units) {
-        int u_next = u + total_warps;
-        if (next_unit) {
-            int t = 0;
-            if (lane == 0)
-                t = atomicAdd(next_unit, 1);
-            u_next = __shfl_sync(0xffffffffu, t, 0);
-        }
-        const int ch = u / sp.groups, g = u - ch * sp.groups;
-        const int j0 = ch * sp.chunk;
-        const int cnt = min(sp.chunk, m - j0);
-        if (ch != staged) {
-            __syncwarp();
-            for (int j = lane; j < cnt; j += 32)
-                spts[j] = COHERENT ? __ldcg(&pts[j0 + j]) : __ldg(&pts[j0 + j]);
-            __syncwarp();
-            staged = ch;
-        }
-        const int i = g * 32 + lane;
-        double S;
-        int nv;
-        fitness_lane<DT, MODE>(V, spts, cnt, fp, i, S, nv);
-        if (i < fp.n) {
-            part_S[(size_t)ch * fp.n + i] = S;
-            part_n[(size_t)ch * fp.n + i] = nv;
-        }
-        u = u_next;
-    }
+    return std::max(1, std::max(std::min(a, (m_max + SMALL_CHUNK - 1) / SMALL_CHUNK), b));
 }
 
 // rho of a particle's total (Eq. normallh, or Eq. ourlh without NORMALIZE).

@@ -40,7 +40,7 @@ __global__ void set_pose_kernel(float *dst, Pose p)
 }
 
 static int mode_of(int flags) { return ((flags & RF_NEAREST) ? 1 : 0) | ((flags & RF_COMPENSATED) ? 0 : 2); }
-static size_t pfo_smem() { return (size_t)FIT_WARPS * CHUNK_MAX * sizeof(float4); }
+static size_t pfo_smem() { return (size_t)FIT_WARPS * sizeof(PairPoints); }
 
 // Largest cooperative grid of the kernel variant (CTAs per SM x SMs).
 static rf_status max_ctas_per_sm(int dtype, int mode, int group, int *per_sm)
@@ -70,15 +70,17 @@ static rf_status check_params(const rf_params *p)
 struct LaunchScratch {
     GridSync *gs = nullptr;
     int *unit_ctr = nullptr;
+    int *hist = nullptr;
     int *block_counts = nullptr;
     double *aps = nullptr;
-    static size_t cleared_bytes() { return sizeof(GridSync) + sizeof(int) * RF_MAX_ITERS; }  // gs and unit_ctr
+    // gs, unit_ctr and hist, in this order: what a launch of B sequences starts from zero
+    static size_t cleared_bytes(int B) { return sizeof(GridSync) + sizeof(int) * ((size_t)RF_MAX_ITERS + (size_t)B * SORT_BUCKETS); }
     rf_status alloc()
     {
         const size_t max_grid = (size_t)MAX_CTAS_PER_SM * sm_count();
-        cudaError_t e = cudaMalloc(&gs, cleared_bytes());
+        cudaError_t e = cudaMalloc(&gs, cleared_bytes(MAX_BATCH));
         if (e == cudaSuccess)
-            unit_ctr = reinterpret_cast<int *>(gs + 1);
+            unit_ctr = reinterpret_cast<int *>(gs + 1), hist = unit_ctr + RF_MAX_ITERS;
         if (e == cudaSuccess)
             e = cudaMalloc(&block_counts, sizeof(int) * MAX_BATCH * max_grid);
         if (e == cudaSuccess)
@@ -93,7 +95,7 @@ struct LaunchScratch {
         cudaFree(block_counts);
         cudaFree(aps);
         gs = nullptr;
-        unit_ctr = block_counts = nullptr;
+        unit_ctr = hist = block_counts = nullptr;
         aps = nullptr;
     }
 };
@@ -117,6 +119,8 @@ struct rf_tracker_s {
     float4 *pts, *cpts;
     double *part_S;
     int *part_n;
+    int *ord;
+    int2 *key;
     int *status;
     float *scale;
     float *pose_ring;   // 2 x 7
@@ -202,6 +206,8 @@ static rf_status fill_problem(rf_tracker tr, const float *depth, const float *pr
     pd.cpts = tr->cpts;
     pd.part_S = tr->part_S;
     pd.part_n = tr->part_n;
+    pd.ord = tr->ord;
+    pd.key = tr->key;
     pd.max_chunks = tr->max_chunks;
     pd.status = tr->status;
     pd.tau = tr->p.tau;
@@ -226,12 +232,13 @@ static rf_status launch_batch(BatchParams &P, const LaunchScratch &ls, int dtype
     const int grid = std::min(use, MAX_CTAS_PER_SM) * sm_count();
     P.gs = ls.gs;
     P.unit_ctr = ls.unit_ctr;
+    P.hist = ls.hist;
     P.block_counts = ls.block_counts;
     P.aps = ls.aps;
     P.k_max_all = 0;
     for (int p = 0; p < P.B; ++p)
         P.k_max_all = std::max(P.k_max_all, P.prob[p].k_max);
-    RF_CUDA(cudaMemsetAsync(ls.gs, 0, LaunchScratch::cleared_bytes(), s));
+    RF_CUDA(cudaMemsetAsync(ls.gs, 0, LaunchScratch::cleared_bytes(P.B), s));
     if (debug_skip) {
         set_int_kernel<<<1, 1, 0, s>>>(&ls.gs->skip, 1);
         RF_CUDA(cudaGetLastError());
@@ -354,6 +361,8 @@ void rf_tracker_destroy(rf_tracker tr)
     cudaFree(tr->cpts);
     cudaFree(tr->part_S);
     cudaFree(tr->part_n);
+    cudaFree(tr->ord);
+    cudaFree(tr->key);
     cudaFree(tr->status);
     cudaFree(tr->scale);
     cudaFree(tr->pose_ring);
@@ -393,7 +402,11 @@ rf_status rf_tracker_create(rf_volume v, const float *pst_dev, int n, const rf_p
         st = tr->ls.alloc();
     cudaError_t e = cudaSuccess;
     if (st == RF_OK) {
-        e = cudaMalloc(&tr->status, sizeof(int));
+        e = cudaMalloc(&tr->ord, sizeof(int) * ((size_t)n + 1));
+        if (e == cudaSuccess)
+            e = cudaMalloc(&tr->key, sizeof(int2) * (size_t)n);
+        if (e == cudaSuccess)
+            e = cudaMalloc(&tr->status, sizeof(int));
         if (e == cudaSuccess)
             e = cudaMalloc(&tr->scale, sizeof(float) * 6);
         if (e == cudaSuccess)

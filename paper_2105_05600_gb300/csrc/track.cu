@@ -2,8 +2,8 @@
 //
 //  rf_depth_to_points   Eq. unproj + stride downsampling (Sec. 4)
 //  rf_overlap_mask      Eq. validness
-//  fitness_eval         Eq. normallh for one PST placement: one warp scores 32
-//                       particles (one per lane) over a chunk of points staged in
+//  fitness_eval         Eq. normallh for one PST placement: one warp scores 64
+//                       particles (two per lane) over a chunk of points staged in
 //                       shared memory, then a fixed-order reduction over chunks
 //  fitness_eval_noalloc the same without device allocation
 //
@@ -19,15 +19,48 @@
 
 namespace rf {
 
+// A CTA takes (point chunk, FIT_WARPS groups of particles) units b, b + gridDim.x,
+// ...: all its warps score the same staged points at the same time and share the
+// neighbourhood's lines through L1, and the next unit's points are loaded while
+// this one is scored.
 template <int DT, int MODE>
-__global__ void __launch_bounds__(FIT_THREADS) fitness_kernel(VolumeDesc V, const float4 *pts, int m, FitParams fp,
-                                                              Split sp, double *part_S, int *part_n)
+__global__ void __launch_bounds__(FIT_THREADS, 2) fitness_kernel(VolumeDesc V, const float4 *pts, int m, FitParams fp,
+                                                                 Split sp, double *part_S, int *part_n)
 {
-    extern __shared__ float4 smem_pts[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int warp_global = blockIdx.x * FIT_WARPS + w;
-    fitness_units<DT, MODE, false>(V, pts, m, fp, sp, part_S, part_n, smem_pts, warp_global, gridDim.x * FIT_WARPS,
-                                   lane, w);
+    __shared__ PairPoints stage[2];
+    static_assert(CHUNK_MAX <= FIT_THREADS, "one point per thread");
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int blocks = (sp.groups + FIT_WARPS - 1) / FIT_WARPS, units = blocks * sp.n_chunks;
+    int u = blockIdx.x;
+    if (u >= units)
+        return;
+    auto load = [&](int unit) {
+        const int j = (unit / blocks) * sp.chunk + tid;
+        return tid < sp.chunk && j < m ? __ldg(&pts[j]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    stage_point(stage[0], tid, load(u));
+    __syncthreads();
+    for (int it = 0; u < units; ++it) {
+        const int next = u + gridDim.x;
+        const float4 np = next < units ? load(next) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int ch = u / blocks, g = (u - ch * blocks) * FIT_WARPS + w;
+        const int cnt = min(sp.chunk, m - ch * sp.chunk);
+        if (g < sp.groups) {
+            const int i[2] = {g * GROUP_PARTICLES + lane, g * GROUP_PARTICLES + 32 + lane};
+            double S[2];
+            int nv[2];
+            fitness_unit<DT, MODE>(V, stage[it & 1], cnt, fp, i, S, nv);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (i[h] < fp.n) {
+                    part_S[(size_t)ch * fp.n + i[h]] = S[h];
+                    part_n[(size_t)ch * fp.n + i[h]] = nv[h];
+                }
+        }
+        stage_point(stage[(it + 1) & 1], tid, np);
+        __syncthreads();
+        u = next;
+    }
 }
 
 // Totals of the chunk partials ([chunk][particle]) and rho.  A block takes 32
@@ -174,10 +207,8 @@ rf_status fitness_eval(rf_volume v, const float *points_dev, int m, const float 
     cudaStream_t s = (cudaStream_t)stream;
     const int mode = mode_of(p->flags);
     FitFn fn = fit_fn(v->d.dtype, mode);
-    const size_t smem = (size_t)FIT_WARPS * CHUNK_MAX * sizeof(float4);
-    RF_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, FIT_THREADS, smem));
+    RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, FIT_THREADS, 0));
     const int grid = std::max(1, per_sm) * sm_count();
     const int total_warps = grid * FIT_WARPS;
     const int max_chunks = max_chunks_for(n, m, total_warps);
@@ -202,7 +233,7 @@ rf_status fitness_eval(rf_volume v, const float *points_dev, int m, const float 
         fp.r[d] = scale[d];
     fp.l1 = (p->flags & RF_L1) != 0;
     fp.right_mult = (p->flags & RF_RIGHT_MULT) != 0;
-    fn<<<grid, FIT_THREADS, smem, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
+    fn<<<grid, FIT_THREADS, 0, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
     RF_CUDA(cudaGetLastError());
     fitness_finish_kernel<<<(n + 31) / 32, FINISH_WARPS * 32, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
                                                           (p->flags & RF_NORMALIZE) != 0, rho_dev, sumsq_dev,
@@ -266,10 +297,8 @@ extern "C" rf_status fitness_eval_noalloc(rf_volume v, const float *points_dev, 
         return st;
     const int mode = mode_of(p->flags);
     FitFn fn = fit_fn(v->d.dtype, mode);
-    const size_t smem = (size_t)FIT_WARPS * CHUNK_MAX * sizeof(float4);
-    RF_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, FIT_THREADS, smem));
+    RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, FIT_THREADS, 0));
     const int grid = std::max(1, per_sm) * sm_count();
     const int total_warps = grid * FIT_WARPS;
     const int cap_chunks = (int)std::min<size_t>(NOALLOC_SCRATCH_BYTES / per_chunk, 1 << 30);
@@ -287,7 +316,7 @@ extern "C" rf_status fitness_eval_noalloc(rf_volume v, const float *points_dev, 
         fp.r[d] = scale[d];
     fp.l1 = (p->flags & RF_L1) != 0;
     fp.right_mult = (p->flags & RF_RIGHT_MULT) != 0;
-    fn<<<grid, FIT_THREADS, smem, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
+    fn<<<grid, FIT_THREADS, 0, s>>>(v->d, (const float4 *)points_dev, m, fp, sp, part_S, part_n);
     RF_CUDA(cudaGetLastError());
     fitness_finish_kernel<<<(n + 31) / 32, FINISH_WARPS * 32, 0, s>>>(n, sp.n_chunks, part_S, part_n, m, p->tau,
                                                           (p->flags & RF_NORMALIZE) != 0, rho_dev, sumsq_dev,

@@ -110,6 +110,30 @@ def test_fitness_ragged_sizes(oracle, nat, m, n):
              rho.cpu().numpy(), S.cpu().numpy(), nv.cpu().numpy())
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i16"])
+@pytest.mark.parametrize("m,n", [(5, 1), (6, 63), (7, 64), (23, 65), (24, 129), (600, 511), (97, 514)])
+def test_fitness_leaving_the_volume(oracle, nat, dtype, m, n):
+    """Particle groups of 64 with a remainder, point batches with a tail, and points far outside the volume or beyond
+    its upper faces next to points inside free, unobserved and surface bricks: every particle against the oracle."""
+    from paper_2105_05600_gb300 import synth
+
+    scene, codes, F64, cfg = analytic_volume_codes("tiny", dtype=dtype)
+    gv = _gpu_volume(nat, cfg, codes)
+    ov = oracle_volume(oracle, cfg, F64)
+    traj = synth.make_trajectory(scene, 2, cfg["speed"], cfg["ang_speed"], cfg["seed"])
+    pts, _, _ = frame_points(oracle, scene, cfg, traj[1])
+    rng = np.random.default_rng(100 * m + n)
+    pts = pts[rng.integers(0, len(pts), m)]
+    pts[::5, :3] *= rng.choice([0.3, 1.5, 4.0, -3.0, 1e4, -1e7], size=(len(pts[::5]), 1))
+    pts = pts.astype(np.float32).astype(np.float64)
+    pst = nat.pst_create(n, seed=4)
+    centre = pose_f32(traj[0])
+    scale = pose_f32([0.1, 0.05, 0.1, 0.4, 0.4, 0.4])[:6]
+    rho, S, nv = nat.fitness_eval(gv, to_gpu_points(pts), pst, centre, scale, nat.make_params())
+    _compare(oracle, ov, pts, pst.cpu().numpy(), range(n), centre, scale, oracle.DEFAULT_FLAGS, 1.0,
+             rho.cpu().numpy(), S.cpu().numpy(), nv.cpu().numpy())
+
+
 @pytest.mark.parametrize("dtype,code,value", [("f32", 0.25, 0.25), ("f16", 0.25, 0.25), ("i16", 8192, 8192 / 32767)])
 def test_constant_volume_closed_form(nat, dtype, code, value):
     import torch
