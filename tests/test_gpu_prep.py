@@ -184,6 +184,49 @@ def test_integrate_parity_many_bricks(oracle, nat):
     np.testing.assert_allclose(Fg[both], ov.F[both], atol=4.0 / 32767)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i16"])
+@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
+    """Volumes on both sides of the brick count from which whole bricks are fused as free space, a frame that ends
+    inside a pixel tile and has holes, and a map that already holds weights up to their limit, unobserved voxels and
+    values other than +1 in front of the surface: values and weights against the oracle after three frames."""
+    import torch
+
+    voxel, trunc = 5.12 / max(dims), 4 * 5.12 / max(dims)
+    scene = synth.make_scene(5.12, 0.3, 11)
+    traj = synth.make_trajectory(scene, 3, 2.0, 2.0, 11)
+    K = synth.intrinsics(97, 61)
+    rng = np.random.default_rng(3)
+    shape = dims[::-1]
+    F0 = np.where(rng.random(shape) < 0.02, rng.uniform(-1, 1, shape), 1.0)
+    F0[:, : dims[1] // 4] = np.where(rng.random((shape[0], dims[1] // 4, shape[2])) < 0.5, np.nan, 1.0)
+    codes0 = synth.encode_values(F0, dtype)
+    W0 = np.where(np.isnan(F0), 0, rng.integers(1, 256, shape)).astype(np.uint8)
+    gv = nat.Volume(dims, voxel, trunc, (0, 0, 0), dtype)
+    gv.upload(codes0, W0)
+    ov = oracle.Volume(dims, voxel, (0, 0, 0), trunc, qmode=dtype)
+    ov.F[:] = synth.decode_values(codes0).reshape(-1)
+    ov.W[:] = W0.reshape(-1)
+    amb = np.zeros(F0.size, bool)
+    for f in range(3):
+        depth = synth.render_depth(scene, traj[f], K, rng)
+        depth[rng.random(depth.shape) < 0.003] = 0.0
+        pose = traj[f].astype(np.float32).astype(np.float64)
+        amb |= ov.integrate_ambiguity(depth, K, pose, tol=1e-4).astype(bool)
+        ov.integrate(depth, K, pose, threads=8)
+        nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
+    codes, W = gv.download()
+    Fg = synth.decode_values(codes).reshape(-1)
+    sure = ~amb
+    assert sure.mean() > 0.98
+    np.testing.assert_array_equal(W.reshape(-1).astype(np.int32)[sure], ov.W[sure])
+    assert np.array_equal(np.isfinite(Fg[sure]), np.isfinite(ov.F[sure]))
+    both = sure & np.isfinite(Fg) & np.isfinite(ov.F)
+    # one rounding step of the storage per frame, FP32 arithmetic (1e-5 of the truncation) below it
+    atol = {"f32": 2e-5, "f16": 3 * 2.0**-11, "i16": 4.0 / 32767}[dtype]
+    np.testing.assert_allclose(Fg[both], ov.F[both], atol=atol)
+
+
 def test_dirty_brick_repacking_matches_full_pack(nat):
     """Fusion repacks only the trilinear cells of bricks it touched; a volume that
     receives the same values by upload (full repack) must score identically."""
