@@ -7,23 +7,31 @@
 // Every product is one launch of umma_gemm_kernel:
 //     C[M x N] = A[M x K] . B[N x K]^T,  A, B bfloat16 row-major (K contiguous),
 //     FP32 accumulation in tensor memory (TMEM), fused epilogue.
-// One CTA owns a 128 x 128 tile of C and 128 TMEM columns:
-//   warp 0, lane 0   TMA producer: 128-row x 64-column slabs of A and B into a
-//                    4-stage shared-memory ring (mbarrier transaction counts)
-//   warp 1, lane 0   MMA issuer: 4 x tcgen05.mma.kind::f16 (M 128, N 128, K 16)
+// One CTA owns a 128 x 32 tile of C and 32 TMEM columns:
+//   warp 0, lane 0   TMA producer: 64-column slabs of A (128 rows) and B (32 rows)
+//                    into an 8-stage shared-memory ring (mbarrier transaction
+//                    counts), one box of 128-byte rows per operand and slab
+//   warp 1, lane 0   MMA issuer: 4 x tcgen05.mma.kind::f16 (M 128, N 32, K 16)
 //                    per slab; tcgen05.commit releases the slab
 //   warps 0..3       epilogue: tcgen05.ld of the warp's 32 accumulator lanes,
 //                    bias / ReLU / gradient mask, bfloat16 or FP32 stores, the
 //                    bfloat16 ones optionally also transposed (the backward
 //                    products reduce over the batch and need batch-contiguous
 //                    operands)
-// Shared-memory operand layout (no swizzle, K-major): the 8 x 8 core matrix of
-// rows 8g..8g+7 and columns 8c..8c+7 of a slab is 128 contiguous bytes at
-// 128 g + 2048 c; one TMA box (8 columns x 128 rows) fills one column group c.
-// So the descriptors' leading-dimension (K) byte offset is 2048 and the
-// stride-dimension (M/N) byte offset is 128; K step j of a slab starts at
-// 4096 j.  Every wait on an mbarrier is bounded in time; on expiry the CTA
-// records RF_ERR_TIMEOUT, lets its copies land, frees its TMEM and returns.
+// The products are tiny (K <= 1024, at most 16 tiles of 128 x 128 at a training batch
+// of 1024), so a launch is bound by its chain of loads, products and epilogue, not by
+// tensor throughput.  Boxes of whole 128-byte rows move a slab in 2 TMA requests of
+// 160 rows; with unswizzled boxes of 16-byte rows the 16 requests of 128 rows were the
+// main loop's limit.  The narrow tile gives four times the CTAs of a 128 x 128 one and
+// a quarter of its epilogue.  Measured, gradient of 512 rows / forward of 1 / 4096
+// rows: 16-byte boxes, 128 x 128 tile 270 / 56 / 62 us; 128-byte boxes, tile N 128:
+// 219 / 38 / 41, N 64: 170 / 30 / 35, N 32: 150 / 29 / 44, N 16: 135 / 27 / 68.
+// Shared-memory operand layout: K-major with the 128-byte swizzle that TMA writes and
+// the MMA reads -- a slab row is 128 bytes, eight rows are one 1024-byte atom, so the
+// stride-dimension (M/N) byte offset is 1024, the leading-dimension offset is unused,
+// tiles are 1024-byte aligned, and K step j of a slab starts 32 j bytes in.  Every wait
+// on an mbarrier is bounded in time; on expiry the CTA records RF_ERR_TIMEOUT, lets its
+// copies land, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -41,18 +49,15 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int GB_M = 128, GB_N = 128, GB_K = 64, GB_STAGES = 4, GB_THREADS = 128;
-constexpr int GB_CHUNK = GB_M * 16;         // one 8-column group of a slab: 128 rows x 16 B
-constexpr int GB_TILE = 8 * GB_CHUNK;       // 16 KiB per operand slab (GB_M == GB_N)
-constexpr int GB_STAGE = 2 * GB_TILE;
-constexpr int GB_LBO = GB_CHUNK;            // K-direction core-matrix step
-constexpr int GB_SBO = 128;                 // M/N-direction core-matrix step
-// A margin after the ring keeps every byte that a descriptor built on these
-// slabs can address inside the allocation, whatever the slab index.
-constexpr int GB_GUARD = 48 * 1024;
-constexpr int GB_BAR_OFF = GB_STAGES * GB_STAGE + GB_GUARD;
-constexpr int GB_SMEM = GB_BAR_OFF + 128 + 1024;  // + barriers, + alignment slack
-constexpr uint32_t GB_TMEM_COLS = 128;
+constexpr int GB_M = 128, GB_N = 32, GB_K = 64, GB_STAGES = 8, GB_THREADS = 128;
+constexpr int GB_ROW = 2 * GB_K;            // bytes of a slab row: one swizzle row
+constexpr int GB_TILE_A = GB_M * GB_ROW, GB_TILE_B = GB_N * GB_ROW;
+constexpr int GB_STAGE = GB_TILE_A + GB_TILE_B;
+constexpr int GB_SBO = 8 * GB_ROW;          // M/N-direction step: eight rows
+constexpr int GB_BAR_OFF = GB_STAGES * GB_STAGE;
+constexpr int GB_SMEM = GB_BAR_OFF + 256 + 1024;  // + barriers, + alignment slack
+constexpr uint32_t GB_TMEM_COLS = 32;
+static_assert(GB_TILE_A % 1024 == 0 && GB_TILE_B % 1024 == 0, "swizzle atoms");
 // kind::f16 instruction descriptor: D FP32 (bits 4-5 = 1), A and B bfloat16
 // (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
 constexpr uint32_t GB_IDESC =
@@ -128,12 +133,11 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: start >> 4 (bits 0-13), leading byte offset
-// >> 4 (16-29), stride byte offset >> 4 (32-45), the fixed 0b001 of bits 46-48,
-// base offset 0, swizzle mode 0 (none, bits 61-63).
+// >> 4 (16-29, unused with a swizzle), stride byte offset >> 4 (32-45), the fixed
+// 0b001 of bits 46-48, base offset 0, swizzle mode 2 (128 bytes, bits 61-63).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
 {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(GB_LBO >> 4) << 16) | ((uint64_t)(GB_SBO >> 4) << 32) |
-           (1ull << 46);
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(GB_SBO >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t acc)
@@ -168,12 +172,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
         v[i] = __uint_as_float(r[i]);
 }
 
-// Column groups of K slab kb that hold data: an even count (whole K steps of 16).
-__device__ __forceinline__ int slab_groups(int K, int kb)
-{
-    const int rem = min(GB_K, K - kb * GB_K);
-    return 2 * ((rem + 15) >> 4);
-}
+// K steps of 16 of slab kb that hold data (the rest of the slab is zero fill).
+__device__ __forceinline__ int slab_steps(int K, int kb) { return (min(GB_K, K - kb * GB_K) + 15) >> 4; }
 
 // ------------------------------------------------------------------ epilogue
 __device__ __forceinline__ void epi_store(const GemmEpi &e, int m, int n, float v[16])
@@ -277,13 +277,10 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                     *s_fail = 1;
                     break;
                 }
-                const int groups = slab_groups(e.K, kb);
-                mbar_expect_tx(bar_full + 8 * s, (uint32_t)(2 * groups * GB_CHUNK));
-                const uint32_t a = base + s * GB_STAGE, b = a + GB_TILE;
-                for (int c = 0; c < groups; ++c) {
-                    tma_load_2d(a + c * GB_CHUNK, &tmA, kb * GB_K + 8 * c, m0, bar_full + 8 * s);
-                    tma_load_2d(b + c * GB_CHUNK, &tmB, kb * GB_K + 8 * c, n0, bar_full + 8 * s);
-                }
+                mbar_expect_tx(bar_full + 8 * s, (uint32_t)GB_STAGE);  // a box counts in full, zero fill included
+                const uint32_t a = base + s * GB_STAGE;
+                tma_load_2d(a, &tmA, kb * GB_K, m0, bar_full + 8 * s);
+                tma_load_2d(a + GB_TILE_A, &tmB, kb * GB_K, n0, bar_full + 8 * s);
                 last[s] = kb;
             }
             // no copy may still be landing when the CTA leaves
@@ -301,11 +298,10 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t a = base + s * GB_STAGE, b = a + GB_TILE;
-                const int steps = slab_groups(e.K, kb) / 2;
+                const uint32_t a = base + s * GB_STAGE, b = a + GB_TILE_A;
+                const int steps = slab_steps(e.K, kb);
                 for (int j = 0; j < steps; ++j)
-                    umma_bf16(tmem, smem_desc(a + j * 2 * GB_CHUNK), smem_desc(b + j * 2 * GB_CHUNK),
-                              (kb | j) != 0 ? 1u : 0u);
+                    umma_bf16(tmem, smem_desc(a + 32 * j), smem_desc(b + 32 * j), (kb | j) != 0 ? 1u : 0u);
                 umma_commit(bar_empty + 8 * s);
             }
             umma_commit(bar_done);  // arrives once every MMA issued above has completed
@@ -492,8 +488,9 @@ rf_status tensor_map_encoder(EncodeTiledFn *out)
 }
 
 // TMA map of a row-major bfloat16 operand [rows x cols] with leading dimension ld:
-// box of 8 columns (16 B) x 128 rows, no swizzle; reads past rows or cols fill 0.
-rf_status operand_map(CUtensorMap *map, const bf16 *ptr, int rows, int cols, int ld)
+// box of 64 columns (128 B) x box_rows rows, 128-byte swizzle; reads past rows or
+// cols fill 0.
+rf_status operand_map(CUtensorMap *map, const bf16 *ptr, int rows, int cols, int ld, int box_rows)
 {
     RF_CHECK_ARG(ptr && ((uintptr_t)ptr & 15) == 0, "operand not 16-byte aligned");
     RF_CHECK_ARG(rows >= 1 && cols >= 1 && ld >= cols && ld % 8 == 0, "operand shape");
@@ -503,10 +500,10 @@ rf_status operand_map(CUtensorMap *map, const bf16 *ptr, int rows, int cols, int
         return st;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(bf16)};
-    const cuuint32_t box[2] = {8, (cuuint32_t)GB_M};
+    const cuuint32_t box[2] = {(cuuint32_t)GB_K, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(ptr), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         set_error("cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -536,9 +533,9 @@ rf_status gemm(const bf16 *A, int lda, const bf16 *B, int ldb, GemmEpi e, cudaSt
     RF_CHECK_ARG(!e.out_h || e.ld_h % 8 == 0, "ld_h");
     RF_CHECK_ARG(!e.out_f || e.ld_f % 4 == 0, "ld_f");
     CUtensorMap ta, tb;
-    rf_status st = operand_map(&ta, A, e.M, e.K, lda);
+    rf_status st = operand_map(&ta, A, e.M, e.K, lda, GB_M);
     if (st == RF_OK)
-        st = operand_map(&tb, B, e.N, e.K, ldb);
+        st = operand_map(&tb, B, e.N, e.K, ldb, GB_N);
     if (st == RF_OK)
         st = gemm_smem_attr();
     if (st != RF_OK)

@@ -89,6 +89,21 @@ def test_forward_dyadic_is_exact(nat, B):
     np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), O)
 
 
+@pytest.mark.parametrize("B", [127, 129, 256])  # one row short of a 128-row tile, one over, two whole tiles
+def test_forward_tile_edges_are_exact(nat, B):
+    import torch
+
+    theta, X = dyadic_problem(21, B)
+    O = assert_exact_premise(theta, X)
+    net = nat.MLP(256)
+    net.set_params(theta.astype(np.float32))
+    out = torch.full((B + 1, mlp.D_OUT_PAD), 7.0, device="cuda")
+    net.forward(to_bf16(X), out=out[:B])
+    assert net.status() == 0
+    np.testing.assert_array_equal(out[:B].cpu().numpy().astype(np.float64), O)
+    assert bool((out[B] == 7.0).all())  # the row after the batch is not written
+
+
 def test_forward_general_within_one_step(nat):
     rng = np.random.default_rng(2)
     theta = mlp.init_params(3)
