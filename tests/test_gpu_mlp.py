@@ -176,6 +176,33 @@ def test_gradient_matches_oracle(nat):
     assert np.all(gv[7][mlp.D_OUT:] == 0.0)
 
 
+@pytest.mark.parametrize("B", [8, 40, 136, 1024])  # the smallest, odd 32-row blocks, over one tile, the largest
+def test_gradient_batch_edges(nat, B):
+    import torch
+
+    theta, X = dyadic_problem(31, B)
+    assert_exact_premise(theta, X)
+    Y = (np.random.default_rng(32).normal(size=(B, 6)) * 0.5).astype(np.float32)
+    L, g_or, O = mlp.loss_and_grad(theta, X, Y.astype(np.float64), round_bf16=True)
+    _, acts = mlp.forward(theta, X, round_bf16=True)
+    Gm = magnitude_gradient(theta, acts, mlp.loss_and_grad_out(O, Y.astype(np.float64), mlp.velocity(acts))[1])
+    net = nat.MLP(B)
+    net.set_params(theta.astype(np.float32))
+    x, y = to_bf16(X), torch.from_numpy(Y).cuda()
+    grad, loss, out = net.gradient(x, y, B)
+    assert net.status() == 0
+    np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), O)
+    assert abs(float(loss.item()) - L) <= 1e-6 * abs(L)
+    assert np.all(np.abs(grad.cpu().numpy() - g_or) <= 4 * U * Gm + 1e-30)
+    # a dataset and result buffers at odd addresses give the same bits
+    x_odd = torch.empty(x.numel() + 1, dtype=x.dtype, device="cuda")[1:].view(x.shape).copy_(x)
+    g_odd, o_odd = (torch.empty(t.numel() + 1, device="cuda")[1:] for t in (grad, out))
+    nat._check(nat.lib.rf_mlp_gradient(net.handle, nat._bf16_ptr(x_odd), nat._dptr(y), None, B, B, nat._dptr(g_odd),
+                                       nat._dptr(loss), nat._dptr(o_odd), nat._stream()))
+    assert net.status() == 0
+    assert torch.equal(g_odd, grad) and torch.equal(o_odd, out.view(-1))
+
+
 def test_gradient_with_index_gather(nat):
     # a permuted batch of a larger dataset gives the gradient of those rows
     import torch
