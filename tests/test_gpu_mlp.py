@@ -89,7 +89,8 @@ def test_forward_dyadic_is_exact(nat, B):
     np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), O)
 
 
-@pytest.mark.parametrize("B", [127, 129, 256])  # one row short of a 128-row tile, one over, two whole tiles
+# the most rows of the small-batch kernel, one over, one short of a 128-row tile, one over, two whole tiles
+@pytest.mark.parametrize("B", [8, 9, 127, 129, 256])
 def test_forward_tile_edges_are_exact(nat, B):
     import torch
 
