@@ -195,11 +195,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
 // K steps of 16 of slab kb that hold data (the rest of the slab is zero fill).
 __device__ __forceinline__ int slab_steps(int K, int kb) { return (min(GB_K, K - kb * GB_K) + 15) >> 4; }
 
-// Programmatic dependent launch: a kernel of a chain waits here for the one before it
-// (whose results are then visible), and lets the next one's blocks start their setup.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // ------------------------------------------------------------------ epilogue
 __device__ __forceinline__ void store_bf16(const GemmEpi &e, int m, int n, const float v[16])
 {
@@ -812,18 +807,8 @@ rf_status gemm_launch(const GemmArgs &a, bool chained, cudaStream_t s)
     rf_status st = gemm_smem_attr();
     if (st != RF_OK)
         return st;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c;
-    memset(&c, 0, sizeof c);
-    c.gridDim = dim3(a.tiles[0] + a.tiles[1] + (a.bias_n + BIAS_CTA_ROWS - 1) / BIAS_CTA_ROWS + (a.loss ? 1 : 0));
-    c.blockDim = dim3(GB_THREADS);
-    c.dynamicSmemBytes = GB_SMEM;
-    c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = chained ? 1 : 0;
-    RF_CUDA(cudaLaunchKernelEx(&c, umma_gemm_kernel, a));
+    const int grid = a.tiles[0] + a.tiles[1] + (a.bias_n + BIAS_CTA_ROWS - 1) / BIAS_CTA_ROWS + (a.loss ? 1 : 0);
+    RF_CUDA(launch_chained(chained, umma_gemm_kernel, grid, GB_THREADS, GB_SMEM, s, a));
     return RF_OK;
 }
 
