@@ -227,6 +227,39 @@ def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
     np.testing.assert_allclose(Fg[both], ov.F[both], atol=atol)
 
 
+@pytest.mark.parametrize("sx,sy", [(1, -1), (-1, 1), (-1, -1)])
+@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
+    """A focal length may have either sign (some datasets publish fy = -480): a fresh map on both sides of the brick
+    count from which whole bricks are fused as free space, unequal focal lengths, two frames, against the oracle."""
+    import torch
+
+    voxel, trunc = 5.12 / max(dims), 4 * 5.12 / max(dims)
+    scene = synth.make_scene(5.12, 0.3, 12)
+    traj = synth.make_trajectory(scene, 2, 2.0, 2.0, 12)
+    K = synth.intrinsics(161, 119)
+    K["fx"], K["fy"] = sx * K["fx"], sy * 1.25 * K["fy"]
+    rng = np.random.default_rng(4)
+    gv = nat.Volume(dims, voxel, trunc, (0, 0, 0), "i16")
+    ov = oracle.Volume(dims, voxel, (0, 0, 0), trunc, qmode="i16")
+    amb = np.zeros(ov.F.size, bool)
+    for f in range(2):
+        depth = synth.render_depth(scene, traj[f], K, rng)
+        depth[7:19, 90:101] = 0.0
+        pose = traj[f].astype(np.float32).astype(np.float64)
+        amb |= ov.integrate_ambiguity(depth, K, pose, tol=1e-4).astype(bool)
+        ov.integrate(depth, K, pose, threads=8)
+        nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
+    codes, W = gv.download()
+    Fg = synth.decode_values(codes).reshape(-1)
+    sure = ~amb
+    assert sure.mean() > 0.98 and ov.W.max() == 2
+    np.testing.assert_array_equal(W.reshape(-1).astype(np.int32)[sure], ov.W[sure])
+    both = sure & np.isfinite(ov.F)
+    assert np.array_equal(np.isfinite(Fg[sure]), np.isfinite(ov.F[sure]))
+    np.testing.assert_allclose(Fg[both], ov.F[both], atol=4.0 / 32767)  # a storage step a frame, FP32 below it
+
+
 def test_dirty_brick_repacking_matches_full_pack(nat):
     """Fusion repacks only the trilinear cells of bricks it touched; a volume that
     receives the same values by upload (full repack) must score identically."""
