@@ -70,17 +70,16 @@ static rf_status check_params(const rf_params *p)
 struct LaunchScratch {
     GridSync *gs = nullptr;
     int *unit_ctr = nullptr;
-    int *hist = nullptr;
     int *block_counts = nullptr;
     double *aps = nullptr;
-    // gs, unit_ctr and hist, in this order: what a launch of B sequences starts from zero
-    static size_t cleared_bytes(int B) { return sizeof(GridSync) + sizeof(int) * ((size_t)RF_MAX_ITERS + (size_t)B * SORT_BUCKETS); }
+    // gs and unit_ctr, in this order: what a launch starts from zero
+    static constexpr size_t CLEARED_BYTES = sizeof(GridSync) + sizeof(int) * RF_MAX_ITERS;
     rf_status alloc()
     {
         const size_t max_grid = (size_t)MAX_CTAS_PER_SM * sm_count();
-        cudaError_t e = cudaMalloc(&gs, cleared_bytes(MAX_BATCH));
+        cudaError_t e = cudaMalloc(&gs, CLEARED_BYTES);
         if (e == cudaSuccess)
-            unit_ctr = reinterpret_cast<int *>(gs + 1), hist = unit_ctr + RF_MAX_ITERS;
+            unit_ctr = reinterpret_cast<int *>(gs + 1);
         if (e == cudaSuccess)
             e = cudaMalloc(&block_counts, sizeof(int) * MAX_BATCH * max_grid);
         if (e == cudaSuccess)
@@ -95,7 +94,7 @@ struct LaunchScratch {
         cudaFree(block_counts);
         cudaFree(aps);
         gs = nullptr;
-        unit_ctr = hist = block_counts = nullptr;
+        unit_ctr = block_counts = nullptr;
         aps = nullptr;
     }
 };
@@ -119,8 +118,8 @@ struct rf_tracker_s {
     float4 *pts, *cpts;
     double *part_S;
     int *part_n;
-    int *ord;
-    int2 *key;
+    int *ord, *key;
+    uint16_t *bucket_counts;
     int *status;
     float *scale;
     float *pose_ring;   // 2 x 7
@@ -208,6 +207,7 @@ static rf_status fill_problem(rf_tracker tr, const float *depth, const float *pr
     pd.part_n = tr->part_n;
     pd.ord = tr->ord;
     pd.key = tr->key;
+    pd.bucket_counts = tr->bucket_counts;
     pd.max_chunks = tr->max_chunks;
     pd.status = tr->status;
     pd.tau = tr->p.tau;
@@ -232,13 +232,12 @@ static rf_status launch_batch(BatchParams &P, const LaunchScratch &ls, int dtype
     const int grid = std::min(use, MAX_CTAS_PER_SM) * sm_count();
     P.gs = ls.gs;
     P.unit_ctr = ls.unit_ctr;
-    P.hist = ls.hist;
     P.block_counts = ls.block_counts;
     P.aps = ls.aps;
     P.k_max_all = 0;
     for (int p = 0; p < P.B; ++p)
         P.k_max_all = std::max(P.k_max_all, P.prob[p].k_max);
-    RF_CUDA(cudaMemsetAsync(ls.gs, 0, LaunchScratch::cleared_bytes(P.B), s));
+    RF_CUDA(cudaMemsetAsync(ls.gs, 0, LaunchScratch::CLEARED_BYTES, s));
     if (debug_skip) {
         set_int_kernel<<<1, 1, 0, s>>>(&ls.gs->skip, 1);
         RF_CUDA(cudaGetLastError());
@@ -363,6 +362,7 @@ void rf_tracker_destroy(rf_tracker tr)
     cudaFree(tr->part_n);
     cudaFree(tr->ord);
     cudaFree(tr->key);
+    cudaFree(tr->bucket_counts);
     cudaFree(tr->status);
     cudaFree(tr->scale);
     cudaFree(tr->pose_ring);
@@ -404,7 +404,9 @@ rf_status rf_tracker_create(rf_volume v, const float *pst_dev, int n, const rf_p
     if (st == RF_OK) {
         e = cudaMalloc(&tr->ord, sizeof(int) * ((size_t)n + 1));
         if (e == cudaSuccess)
-            e = cudaMalloc(&tr->key, sizeof(int2) * (size_t)n);
+            e = cudaMalloc(&tr->key, sizeof(int) * (size_t)n);
+        if (e == cudaSuccess)
+            e = cudaMalloc(&tr->bucket_counts, sizeof(uint16_t) * SORT_BUCKETS * (((size_t)n + SORT_BLOCK - 1) / SORT_BLOCK));
         if (e == cudaSuccess)
             e = cudaMalloc(&tr->status, sizeof(int));
         if (e == cudaSuccess)

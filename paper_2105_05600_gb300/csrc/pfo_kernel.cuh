@@ -25,9 +25,13 @@ rf_status launch_integrate_dev(const VolumeDesc &V, const float *depth, const In
 
 constexpr int SORT_BITS = 10;
 constexpr int SORT_BUCKETS = 1 << SORT_BITS;
-// Lookups an iteration from which the scoring order pays for itself (it costs about 4 us
-// an iteration): at 9.8 M a frame takes 615 us without and 637 us with it, at 19 M 926 and
-// 950, at 21 M (float) 1420 and 1297, at 26 M 1307 and 1281.
+constexpr int SORT_BLOCK = 512;  // particles that one CTA ranks together
+// Lookups an iteration (particles x points of the level) from which the scoring order pays
+// for itself.  Frames of ten iterations with the order against without it, 64^3 float, 256^3
+// and 512^3 int16 and 384^3 half maps, two rooms each, mean (range): 4.9 M lookups 0.990
+// (0.97 .. 1.01) times as fast, 9.8 M 0.995, 14.7 M 0.993, 19.7 M 1.008 (0.97 .. 1.06),
+// 39 M 1.014 (0.96 .. 1.07), 59 M 1.017 (0.99 .. 1.07): wide swarms gain, tight ones lose
+// its 2 to 4 us an iteration, and the mean crosses 1 between 14.7 M and 19.7 M.
 constexpr long long SORT_MIN_WORK = 1ll << 24;
 
 // ------------------------------------------------------------------ launch descriptors
@@ -50,8 +54,9 @@ struct ProblemDesc {
     double *part_S;
     int *part_n;
     int max_chunks;
-    int *ord;   // [n_tmpl] particles in scoring order, rebuilt every iteration; ord[n_tmpl] = place of particle 0
-    int2 *key;  // [n_tmpl] (bucket, place in it) of each particle
+    int *ord;  // [n_tmpl] particles in scoring order, rebuilt every iteration; ord[n_tmpl] = place of particle 0
+    int *key;  // [n_tmpl] bucket | place among its block's particles of the bucket << SORT_BITS
+    uint16_t *bucket_counts;  // [blocks of SORT_BLOCK particles][SORT_BUCKETS]
     int *status;
     float tau, beta, eps, stop_eps;
     int k_max, flags;
@@ -68,9 +73,8 @@ struct BatchParams {
     int B;
     int k_max_all;
     int work_warps;
-    GridSync *gs;       // gs, unit_ctr and hist are one allocation, zero at launch
+    GridSync *gs;       // gs and unit_ctr are one allocation, zero at launch
     int *unit_ctr;      // [RF_MAX_ITERS]
-    int *hist;          // [MAX_BATCH][SORT_BUCKETS]
     int *block_counts;  // [grid][MAX_BATCH]
     double *aps;        // [grid][MAX_BATCH][APW]
     long long timeout_ns;
@@ -190,8 +194,10 @@ __device__ __forceinline__ double warp_sum8(double v[8], int lane)
 // Scoring order.  A warp scores particles that are neighbours in the swarm, so
 // that its lanes look up neighbouring cells.  The swarm is an anisotropic ball;
 // splitting the axis of the largest remaining extent in two, SORT_BITS times,
-// gives buckets of about equal sides.  Every particle's sum is the same in any order;
-// 20,000 particles of random order cost 4 to 16 % more per lookup.
+// gives buckets of about equal sides.  20,000 particles of random order cost 4 to 16 %
+// more per lookup.  The order is a stable counting sort, buckets first and particle
+// indices inside a bucket, so it is a function of the swarm alone and every sum that
+// follows it is the same in every run and for every grid.
 // split[s] = axis | depth << 8.
 __device__ __forceinline__ void sort_splits(const float r[6], int split[SORT_BITS])
 {
@@ -225,6 +231,118 @@ __device__ __forceinline__ int sort_key(const float *pst, int ld, int i, const i
     return key;
 }
 
+// First pass of the sort, one block of SORT_BLOCK particles by one CTA: every particle's
+// bucket, its place among the block's earlier particles of that bucket, and the block's
+// counts.  A warp takes consecutive particles, 32 at a time, and counts them in its own
+// row of `rows` (FIT_WARPS x SORT_BUCKETS, shared memory); the particles of a round that
+// share a bucket find each other by __match_any_sync, so no place depends on the order of
+// arrival.
+// Bound by latency: loads, SORT_ROUNDS dependent rounds and the prefix.  Blocks of 512
+// particles, ranked beside the point tests by CTAs that take no points: 10,000 / 20,000
+// particle frames 2519 / 14275 us; blocks of 1024 2541 / 14423, of 256 2519 / 14311.  Global
+// counters with atomic arrival order took 2533 / 14407 us and ranked a bucket's particles
+// differently in every run.
+constexpr int SORT_ROUNDS = SORT_BLOCK / FIT_THREADS;
+static __device__ void sort_count(const ProblemDesc &pd, int n, int blk, const int split[SORT_BITS], uint16_t *rows)
+{
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    __syncthreads();
+    for (int q = tid; q < FIT_WARPS * SORT_BUCKETS / 8; q += FIT_THREADS)
+        reinterpret_cast<uint4 *>(rows)[q] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    uint16_t *row = rows + w * SORT_BUCKETS;
+    const int i0 = blk * SORT_BLOCK + w * (SORT_BLOCK / FIT_WARPS) + lane;
+    int key[SORT_ROUNDS], place[SORT_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SORT_ROUNDS; ++r)
+        key[r] = i0 + 32 * r < n ? sort_key(pd.pst, pd.n_tmpl, i0 + 32 * r, split) : -1;
+#pragma unroll
+    for (int r = 0; r < SORT_ROUNDS; ++r) {
+        const unsigned same = __match_any_sync(0xffffffffu, key[r]);
+        const unsigned before = same & ((1u << lane) - 1u);
+        const int old = key[r] >= 0 ? row[key[r]] : 0;
+        place[r] = old + __popc(before);
+        __syncwarp();
+        if (key[r] >= 0 && before == 0u)
+            row[key[r]] = (uint16_t)(old + __popc(same));
+        __syncwarp();
+    }
+    __syncthreads();
+    // four buckets a thread: a warp's row becomes the counts of the warps before it
+    unsigned c[4] = {0u, 0u, 0u, 0u};
+    for (int q = 0; q < FIT_WARPS; ++q) {
+        uint2 *at = reinterpret_cast<uint2 *>(rows + q * SORT_BUCKETS) + tid;
+        const uint2 v = *at;
+        *at = make_uint2(c[0] | c[1] << 16, c[2] | c[3] << 16);
+        c[0] += v.x & 0xFFFFu;
+        c[1] += v.x >> 16;
+        c[2] += v.y & 0xFFFFu;
+        c[3] += v.y >> 16;
+    }
+    reinterpret_cast<uint2 *>(pd.bucket_counts + (size_t)blk * SORT_BUCKETS)[tid] =
+        make_uint2(c[0] | c[1] << 16, c[2] | c[3] << 16);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SORT_ROUNDS; ++r)
+        if (key[r] >= 0)
+            pd.key[i0 + 32 * r] = key[r] | (place[r] + row[key[r]]) << SORT_BITS;
+}
+
+// Second pass, after a grid barrier: the same block's particles to their places, which
+// follow the smaller buckets, then the bucket's particles of the blocks before.
+// `at` holds SORT_BUCKETS + FIT_WARPS ints of shared memory.
+static __device__ void sort_place(const ProblemDesc &pd, int n, int blk, int *at)
+{
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int n_blocks = (n + SORT_BLOCK - 1) / SORT_BLOCK;
+    const int i0 = blk * SORT_BLOCK + tid;
+    int kp[SORT_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SORT_ROUNDS; ++r)
+        kp[r] = i0 + FIT_THREADS * r < n ? __ldcg(&pd.key[i0 + FIT_THREADS * r]) : 0;
+    int all[4] = {0, 0, 0, 0}, before[4] = {0, 0, 0, 0};
+#pragma unroll 8
+    for (int q = 0; q < n_blocks; ++q) {
+        const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(pd.bucket_counts + (size_t)q * SORT_BUCKETS) + tid);
+        const int c[4] = {(int)(v.x & 0xFFFFu), (int)(v.x >> 16), (int)(v.y & 0xFFFFu), (int)(v.y >> 16)};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            all[e] += c[e];
+            before[e] += q < blk ? c[e] : 0;
+        }
+    }
+    const int mine = all[0] + all[1] + all[2] + all[3];
+    int inc = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, inc, o);
+        inc += lane >= o ? up : 0;
+    }
+    int *warp_sum = at + SORT_BUCKETS;
+    __syncthreads();
+    if (lane == 31)
+        warp_sum[w] = inc;
+    __syncthreads();
+    int first = inc - mine;
+    for (int q = 0; q < w; ++q)
+        first += warp_sum[q];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        at[4 * tid + e] = first + before[e];
+        first += all[e];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SORT_ROUNDS; ++r) {
+        const int i = i0 + FIT_THREADS * r;
+        if (i < n) {
+            const int slot = at[kp[r] & (SORT_BUCKETS - 1)] + (kp[r] >> SORT_BITS);
+            pd.ord[slot] = i;
+            if (i == 0)
+                pd.ord[pd.n_tmpl] = slot;
+        }
+    }
+}
+
 // Per-sequence state, identical in every CTA (computed redundantly in a fixed order).
 struct PState {
     Pose c, prev;
@@ -252,8 +370,11 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
     __shared__ int red_i[3];
     static_assert(FIT_WARPS == 8, "phase C: one warp per APS quantity");
     __shared__ int s_total_units;
-    __shared__ int bucket_at[SORT_BUCKETS];
-    static_assert(SORT_BUCKETS == 4 * FIT_THREADS, "one int4 of buckets per thread");
+    static_assert(SORT_BUCKETS == 4 * FIT_THREADS, "four buckets per thread");
+    static_assert(SORT_BLOCK == SORT_ROUNDS * FIT_THREADS, "whole rounds of a block");
+    static_assert(FIT_WARPS * SORT_BUCKETS * sizeof(uint16_t) <= FIT_WARPS * sizeof(PairPoints) &&
+                      (SORT_BUCKETS + FIT_WARPS) * sizeof(int) <= FIT_WARPS * sizeof(PairPoints),
+                  "the sort works in the points' shared memory");
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int G = gridDim.x, b = blockIdx.x;
@@ -333,17 +454,36 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 sort_splits(s.r, s.split);
         }
         __syncthreads();
-        int T = 0;
+        int T = 0, sort_blocks = 0;
         bool any = false;
         for (int p = 0; p < B; ++p)
             if (st[p].active) {
                 any = true;
                 T += st[p].m_lvl;
+                sort_blocks += st[p].sorted ? (st[p].n_lvl + SORT_BLOCK - 1) / SORT_BLOCK : 0;
             }
         if (!any)
             break;  // identical decision in every CTA
+        // The last CTAs order the swarms, one block of particles each, while the others take the
+        // points: neither waits for the other.
+        const int n_sort = min(sort_blocks, G / 2);
+        auto each_block = [&](auto &&f) {
+            if (b < G - n_sort)
+                return;
+            for (int q = G - 1 - b; q < sort_blocks; q += n_sort) {
+                int p = 0, blk = q;
+                for (;; ++p) {
+                    const int n = st[p].sorted ? (st[p].n_lvl + SORT_BLOCK - 1) / SORT_BLOCK : 0;
+                    if (blk < n)
+                        break;
+                    blk -= n;
+                }
+                if (st[p].active)
+                    f(P.prob[p], st[p], blk);
+            }
+        };
         // ---- phase A: overlap counts per (CTA, sequence) over the concatenated point sets
-        const int seg = (T + G - 1) / G;
+        const int seg = (T + G - n_sort - 1) / (G - n_sort);
         const int jb = min(T, b * seg), je = min(T, jb + seg);
         {
             int base = 0;
@@ -377,14 +517,9 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 base += st[p].m_lvl;
             }
         }
-        for (int p = 0; p < B; ++p)
-            if (st[p].active && st[p].sorted) {
-                const ProblemDesc &pd = P.prob[p];
-                for (int i = b * blockDim.x + tid; i < st[p].n_lvl; i += G * blockDim.x) {
-                    const int key = sort_key(pd.pst, pd.n_tmpl, i, st[p].split);
-                    pd.key[i] = make_int2(key, atomicAdd(&P.hist[p * SORT_BUCKETS + key], 1));
-                }
-            }
+        each_block([&](const ProblemDesc &pd, const PState &s, int blk) {
+            sort_count(pd, s.n_lvl, blk, s.split, reinterpret_cast<uint16_t *>(smem_raw));
+        });
         if (!grid_barrier(P, n_barriers))
             return;
         // ---- phase A': per-sequence offsets and |O_k|, then the compaction
@@ -457,37 +592,9 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
                 base += st[p].m_lvl;
             }
         }
-        for (int p = 0; p < B; ++p) {
-            if (!st[p].active || !st[p].sorted || b * (int)blockDim.x >= st[p].n_lvl)
-                continue;
-            const ProblemDesc &pd = P.prob[p];
-            // first place of each bucket: exclusive scan of the counts
-            const int4 c = __ldcg(reinterpret_cast<const int4 *>(P.hist + p * SORT_BUCKETS) + tid);
-            const int mine = c.x + c.y + c.z + c.w;
-            int inc = mine;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int up = __shfl_up_sync(0xffffffffu, inc, o);
-                inc += lane >= o ? up : 0;
-            }
-            __syncthreads();
-            if (lane == 31)
-                warp_tot[w] = inc;
-            __syncthreads();
-            int at = inc - mine;
-            for (int q = 0; q < w; ++q)
-                at += warp_tot[q];
-            bucket_at[4 * tid] = at;
-            bucket_at[4 * tid + 1] = at + c.x;
-            bucket_at[4 * tid + 2] = at + c.x + c.y;
-            bucket_at[4 * tid + 3] = at + c.x + c.y + c.z;
-            __syncthreads();
-            for (int i = b * blockDim.x + tid; i < st[p].n_lvl; i += G * blockDim.x) {
-                const int2 kp = __ldcg(&pd.key[i]);
-                pd.ord[bucket_at[kp.x] + kp.y] = i;
-                if (i == 0)
-                    pd.ord[pd.n_tmpl] = bucket_at[kp.x] + kp.y;
-            }
-        }
+        each_block([&](const ProblemDesc &pd, const PState &s, int blk) {
+            sort_place(pd, s.n_lvl, blk, reinterpret_cast<int *>(smem_raw));
+        });
         if (!grid_barrier(P, n_barriers))
             return;
         // ---- phase B: fitness of every particle of every active sequence (Eq. normallh)
@@ -562,9 +669,6 @@ __global__ void __launch_bounds__(FIT_THREADS, RF_PFO_MIN_BLOCKS) pfo_batch_kern
         }
         if (!grid_barrier(P, n_barriers))
             return;
-        if (b == 0)  // the sort's counts, for the next iteration
-            for (int q = tid; q < B * SORT_BUCKETS; q += blockDim.x)
-                P.hist[q] = 0;
         // ---- phase B': per-particle totals, rho, per-CTA APS sums (Eq. ebs, Eq. wafit)
         for (int p = 0; p < B; ++p) {
             if (!st[p].active)

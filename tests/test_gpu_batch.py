@@ -135,6 +135,19 @@ def test_batch_equals_sequences_alone(nat, use_graph):
             assert sa[i][f] == sb[i][f]
 
 
+def test_batch_of_ordered_swarms_equals_sequences_alone(nat):
+    # swarms large enough to be scored in an order of their own, next to one that is not
+    big = dict(dims=64, voxel=0.04, w=80, h=60, n=4096, k_max=6, stride=1, seed=3, frames=3)
+    specs = [big, dict(SPECS[1], frames=3), dict(big, w=96, h=72, n=3001, voxel=0.05, seed=4)]
+    pa, sa = _run_alone(nat, specs)
+    for use_graph in (False, True):
+        pb, sb, _ = _run_batch(nat, specs, use_graph)
+        for i in range(len(specs)):
+            for f in range(len(pa[i])):
+                np.testing.assert_array_equal(pa[i][f], pb[i][f])
+                assert sa[i][f] == sb[i][f]
+
+
 def _analytic_batch(oracle, nat, specs, use_graph, autotune):
     """Each spec's volume holds its room's analytic TSDF (also given to the oracle);
     frame 0 is fused as an all-invalid depth map, which changes no voxel, so the

@@ -315,6 +315,62 @@ def test_tracker_is_deterministic(oracle, nat):
     assert out[0][1] == out[1][1]
 
 
+# a remainder of a block of 512 ordered particles, two whole blocks, one particle over, a remainder of a warp
+@pytest.mark.parametrize("n", [874, 1024, 1025, 2100])
+def test_tracker_parity_ordered_swarm(oracle, nat, n):
+    """Frames of 160 x 120 points, from 2^24 lookups an iteration, whose swarm is scored in an order of its own."""
+    import torch
+
+    scene, codes, F64, cfg = analytic_volume_codes("tiny", dtype="i16")
+    gv = nat.Volume(cfg["dims"], cfg["voxel"], cfg["trunc"], (0, 0, 0), "i16")
+    gv.upload(codes)
+    ov = oracle_volume(oracle, cfg, F64)
+    traj = synth.make_trajectory(scene, 2, cfg["speed"], cfg["ang_speed"], cfg["seed"])
+    K = synth.intrinsics(160, 120)
+    d0, d1 = (synth.render_depth(scene, traj[f], K) for f in range(2))
+    assert n * 160 * 120 >= 1 << 24
+    tr = nat.Tracker(gv, nat.pst_create(n, seed=1), nat.make_params(k_max=3), 160, 120)
+    tr.set_scale([0.1] * 6)
+    prev = pose_f32(traj[0])
+    pose, gst, status = nat.pfo_track_frame(tr, torch.from_numpy(d1).cuda(), torch.from_numpy(d0).cuda(), K, prev)
+    assert status == 0
+    _check_frame(oracle, ov, gst, pose, [(oracle.unproject(d1, K, 1), n)], d0, K, prev, prev,
+                 np.full(6, np.float32(0.1)), n, _oracle_params(oracle, 3), tr)
+
+
+def test_scoring_order_is_fixed(nat):
+    """4096 particles x 4800 points: the swarm is scored in an order of its own, which must be the same in every run.
+    The map depends on z alone and the template has no rotations and mirrored pairs (w_x, w_y, w_z), (-w_x, -w_y, w_z),
+    so a pair's weights are equal and the x and y sums of Eq. ebs cancel exactly: what is left of them is the rounding
+    of the FP64 additions, in which any change of their order shows at once.  All frames must agree in every bit."""
+    import torch
+
+    dims, voxel, trunc, n = 64, 0.04, 0.12, 4096
+    z = (np.arange(dims) + 0.5) * voxel
+    F = np.broadcast_to(np.clip((1.7 - z) / trunc, -1, 1)[:, None, None], (dims,) * 3)
+    gv = nat.Volume(dims, voxel, trunc, (0, 0, 0), "f32")
+    gv.upload(synth.encode_values(F, "f32"))
+    w = np.random.default_rng(6).uniform(-0.6, 0.6, (n // 2, 3))
+    pst = np.zeros((6, n), np.float32)
+    pst[3:, 0::2] = w.T
+    pst[3:, 1::2] = w.T * np.array([[-1], [-1], [1]])
+    pst[:, 0] = pst[:, 1] = 0.0  # particle 0 is the centre
+    K = synth.intrinsics(80, 60)
+    depth = torch.full((60, 80), 1.15, device="cuda")
+    tr = nat.Tracker(gv, torch.from_numpy(pst).cuda(), nat.make_params(k_max=1), 80, 60)
+    first = None
+    for _ in range(24):
+        tr.set_scale([0.1] * 6)
+        pose, gst, status = nat.pfo_track_frame(tr, depth, depth, K, [1, 0, 0, 0, 1.28, 1.28, 0.5])
+        assert status == 0
+        row = gst["it"][0]
+        assert gst["n_points"] * n >= 1 << 24 and row["n_overlap"] > 3000 and row["n_aps"] > n // 8
+        off = np.abs(row["offset"])
+        assert off[5] > 1e-3 and max(off[3:5]) < 1e-12 * off[5]  # z moves; x and y are rounding
+        first = first or (pose.tolist(), gst)
+        assert first == (pose.tolist(), gst)
+
+
 def test_sequence_mode_matches_explicit_calls(oracle, nat):
     import torch
 
