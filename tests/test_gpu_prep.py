@@ -260,6 +260,44 @@ def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
     np.testing.assert_allclose(Fg[both], ov.F[both], atol=4.0 / 32767)  # a storage step a frame, FP32 below it
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+def test_integrate_keeps_infinities(nat, dtype, dims):
+    """Values that a float or half map can hold but no frame produces: the running average (W F + 1) / (W + 1) as IEEE
+    arithmetic gives it, in free bricks, in bricks next to invalid pixels and on small maps."""
+    import torch
+
+    voxel = 5.12 / max(dims)
+    np_t = np.float32 if dtype == "f32" else np.float16
+    special = [np.inf, -np.inf] + ([3e38, -3e38, 1e-40, -1e-45, 1e31] if dtype == "f32" else [65504, -65504, 6e-8])
+    rng = np.random.default_rng(5)
+    shape = dims[::-1]
+    F0 = np.ones(shape, np_t)
+    at = rng.random(shape) < 0.01
+    F0[at] = rng.choice(np.array(special, np_t), at.sum())
+    W0 = rng.integers(1, 200, shape).astype(np.uint8)
+    gv = nat.Volume(dims, voxel, 3 * voxel, (0, 0, 0), dtype)
+    gv.upload(F0, W0)
+    K = synth.intrinsics(160, 120, z_max=9.0)
+    depth = np.full((120, 160), 8.5, np.float32)  # beyond the map: f = 1 in every voxel in view
+    depth[50:60, 70:75] = 0.0
+    nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, [1, 0, 0, 0, 2.5, 2.5, -1.0])
+    F1, W1 = gv.download()
+    F1, W1 = F1.reshape(shape), W1.reshape(shape)
+    up = W1 == W0 + 1
+    assert np.array_equal(W1[~up], W0[~up]) and up.mean() > 0.3 and up[at].sum() > 1000
+    np.testing.assert_array_equal(F1[~up], F0[~up])
+    w, one = W0[up].astype(np.float32), np.float32(1)
+    with np.errstate(over="ignore"):
+        # one rounding of W F + 1 to FP32, as fma does: W F is exact in FP64, and where the 1 lies below its last bit
+        # the next FP64 number stands for it (it decides ties of the FP32 rounding)
+        total = w.astype(np.float64) * F0[up].astype(np.float64)
+        total = np.where(np.isfinite(total) & (np.abs(total) > 2.0**53), np.nextafter(total, np.inf), total + 1.0)
+        total = total.astype(np.float32)
+        want = (total / (w + one)).astype(np_t)
+    np.testing.assert_array_equal(F1[up], want)
+
+
 def test_dirty_brick_repacking_matches_full_pack(nat):
     """Fusion repacks only the trilinear cells of bricks it touched; a volume that
     receives the same values by upload (full repack) must score identically."""
