@@ -50,6 +50,15 @@ rf_status rf_l2_gather_probe(const void *buf_dev, size_t bytes, int loads_per_th
  */
 rf_status rf_volume_counters(rf_volume v, long long out_host[3], int reset);
 
+/*
+ * rf_quotient_probe -- the quotients of tsdf_integrate by themselves, so that they
+ * can be held against IEEE division: out[i] = a[i] / b[i], or 1 / b[i] when a_dev
+ * is NULL, for operands and quotients in the normal range of float.
+ *   a_dev (or NULL), b_dev, out_dev   device float[n], n >= 1
+ * Asynchronous.
+ */
+rf_status rf_quotient_probe(const float *a_dev, const float *b_dev, size_t n, float *out_dev, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -102,7 +102,7 @@ EXPORTS = ["rf_last_error", "rf_version", "pst_create", "rf_volume_create", "rf_
            "rf_proposal_default_params", "rf_proposal_apply", "rf_learned_create", "rf_learned_destroy",
            "rf_learned_start", "rf_learned_step", "rf_l2_gather_probe", "rf_volume_counters",
            "rf_tracker_set_config", "rf_tracker_get_config", "rf_tracker_autotune", "rf_mlp_evaluate",
-           "rf_mlp_calibrate_scale"]
+           "rf_mlp_calibrate_scale", "rf_quotient_probe"]
 
 
 def _load():
@@ -178,6 +178,7 @@ def _load():
         "rf_learned_step": (i, [P, P, i, ctypes.POINTER(rf_intrinsics), i, ctypes.POINTER(rf_pose), P, P, P]),
         "rf_l2_gather_probe": (i, [P, ctypes.c_size_t, i, i, i, P, P]),
         "rf_volume_counters": (i, [P, ctypes.POINTER(ctypes.c_longlong), i]),
+        "rf_quotient_probe": (i, [P, P, ctypes.c_size_t, P, P]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
@@ -834,3 +835,11 @@ def rf_l2_gather_probe(buf, loads_per_thread, ctas_per_sm, sink, mode=0, stream=
     tensor of ctas_per_sm x SMs x 256 entries."""
     _check(lib.rf_l2_gather_probe(_dptr(buf), buf.numel() * buf.element_size(), int(loads_per_thread),
                                   int(ctas_per_sm), int(mode), _dptr(sink), _stream(stream)))
+
+
+def rf_quotient_probe(a, b, out, stream=None):
+    """The fusion's quotient a / b (1 / b when a is None) of CUDA float tensors, into out."""
+    import torch
+
+    _check(lib.rf_quotient_probe(None if a is None else _dptr(a, torch.float32), _dptr(b, torch.float32), b.numel(),
+                                 _dptr(out, torch.float32), _stream(stream)))

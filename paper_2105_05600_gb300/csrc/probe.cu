@@ -1,5 +1,6 @@
 // probe.cu -- the gather microbenchmark that gives the fitness lookups their
-// roofline (rf_l2_gather_probe, include/rf_measure.h).
+// roofline, and the fusion's quotients on their own (rf_l2_gather_probe,
+// rf_quotient_probe, include/rf_measure.h).
 #include "common.cuh"
 #include "fitness.cuh"
 #include "rf_measure.h"
@@ -45,6 +46,14 @@ __global__ void __launch_bounds__(256) l2_gather_probe_kernel(const uint4 *__res
     sink[gtid] = acc;
 }
 
+__global__ void __launch_bounds__(256) quotient_probe_kernel(const float *a, const float *b, size_t n, float *out)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const float y = recip(b[i]);
+        out[i] = a ? div_by(a[i], b[i], y) : y;
+    }
+}
+
 }  // namespace rf
 
 using namespace rf;
@@ -66,6 +75,15 @@ extern "C" rf_status rf_l2_gather_probe(const void *buf_dev, size_t bytes, int l
     l2_gather_probe_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const uint4 *>(buf_dev),
                                                                     (uint32_t)(bytes / 16), loads_per_thread, mode,
                                                                     sink_dev);
+    RF_CUDA(cudaGetLastError());
+    return RF_OK;
+}
+
+extern "C" rf_status rf_quotient_probe(const float *a_dev, const float *b_dev, size_t n, float *out_dev, void *stream)
+{
+    RF_CHECK_ARG(b_dev && out_dev, "null pointer");
+    RF_CHECK_ARG(n >= 1, "n must be >= 1");
+    quotient_probe_kernel<<<8 * sm_count(), 256, 0, (cudaStream_t)stream>>>(a_dev, b_dev, n, out_dev);
     RF_CUDA(cudaGetLastError());
     return RF_OK;
 }

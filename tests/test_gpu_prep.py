@@ -298,6 +298,53 @@ def test_integrate_keeps_infinities(nat, dtype, dims):
     np.testing.assert_array_equal(F1[up], want)
 
 
+def _hard_quotients(n, rng):
+    """Pairs (a, b) of 24-bit integers whose quotient lies next to a midpoint of two floats: a 2^k = b m + c with m an
+    odd 25-bit integer and c a few units, k = 24 or 25."""
+    A, B = [], []
+    while sum(map(len, A)) < n:
+        b = (rng.integers(1 << 23, 1 << 24, 1 << 20) | 1).astype(np.uint64)
+        b[::8] = (1 << 24) - 1 - 2 * rng.integers(0, 64, len(b[::8])).astype(np.uint64)
+        c = rng.choice(np.array([-4, -3, -2, -1, 1, 2, 3, 4]), b.size)
+        k = rng.integers(24, 26, b.size).astype(np.uint64)
+        mod = np.uint64(1) << k
+        inv = np.ones_like(b)
+        for _ in range(6):
+            inv = inv * (np.uint64(2) - b * inv)  # the inverse of an odd b modulo 2^64, by Newton
+        m = ((-c).astype(np.uint64) * inv) & (mod - np.uint64(1))
+        m = np.where(m < 1 << 24, m + mod, m)
+        a2 = b * m + c.astype(np.uint64)
+        a = a2 >> k
+        ok = (m & np.uint64(1) == 1) & (m < 1 << 25) & (a << k == a2) & (a >= 1 << 23) & (a < 1 << 24)
+        A.append(a[ok])
+        B.append(b[ok])
+    return np.concatenate(A)[:n].astype(np.float32), np.concatenate(B)[:n].astype(np.float32)
+
+
+def test_fusion_quotients_are_those_of_ieee_division(nat):
+    """Every significand's reciprocal, and quotients that a last-bit error anywhere would round the wrong way:
+    next to midpoints, the running average's divisors 1 .. 256, depths over a wide range."""
+    import torch
+
+    rng = np.random.default_rng(8)
+    b = (np.arange(1 << 23, dtype=np.uint32) | np.uint32(127 << 23)).view(np.float32)
+    scale = np.float32(2.0) ** rng.integers(-29, 30, b.size).astype(np.float32)
+    dev = lambda x: torch.from_numpy(x).cuda()
+    for bs in (b, b * scale):
+        out = torch.empty(b.size, device="cuda")
+        nat.rf_quotient_probe(None, dev(bs), out)
+        np.testing.assert_array_equal(out.cpu().numpy(), np.float32(1) / bs)
+    hard = _hard_quotients(1 << 20, rng)
+    div = np.repeat(np.arange(1, 257, dtype=np.float32), 4096)
+    avg = ((div - 1) * rng.uniform(-1, 1, div.size) + rng.uniform(-1, 1, div.size)).astype(np.float32)
+    z = np.exp(rng.uniform(np.log(1e-8), np.log(1e4), 1 << 20)).astype(np.float32)
+    nu = (rng.normal(size=z.size) * z * 500).astype(np.float32)
+    for a, d in (hard, (hard[0] * np.float32(2.0**-9), hard[1] * np.float32(2.0**-22)), (avg, div), (nu, z)):
+        out = torch.empty(a.size, device="cuda")
+        nat.rf_quotient_probe(dev(a), dev(d), out)
+        np.testing.assert_array_equal(out.cpu().numpy(), a / d)
+
+
 def test_dirty_brick_repacking_matches_full_pack(nat):
     """Fusion repacks only the trilinear cells of bricks it touched; a volume that
     receives the same values by upload (full repack) must score identically."""
