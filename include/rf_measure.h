@@ -51,6 +51,13 @@ rf_status rf_l2_gather_probe(const void *buf_dev, size_t bytes, int loads_per_th
 rf_status rf_volume_counters(rf_volume v, long long out_host[3], int reset);
 
 /*
+ * rf_volume_fusion_lists -- how the last tsdf_integrate took the bricks that passed
+ * its frustum test: out_host[0] projected voxel by voxel, out_host[1] fused as free
+ * space as a whole (volumes of 16,384 bricks and more).  Synchronises the device.
+ */
+rf_status rf_volume_fusion_lists(rf_volume v, int out_host[2]);
+
+/*
  * rf_quotient_probe -- the quotients of tsdf_integrate by themselves, so that they
  * can be held against IEEE division: out[i] = a[i] / b[i], or 1 / b[i] when a_dev
  * is NULL, for operands and quotients in the normal range of float.

@@ -102,7 +102,7 @@ EXPORTS = ["rf_last_error", "rf_version", "pst_create", "rf_volume_create", "rf_
            "rf_proposal_default_params", "rf_proposal_apply", "rf_learned_create", "rf_learned_destroy",
            "rf_learned_start", "rf_learned_step", "rf_l2_gather_probe", "rf_volume_counters",
            "rf_tracker_set_config", "rf_tracker_get_config", "rf_tracker_autotune", "rf_mlp_evaluate",
-           "rf_mlp_calibrate_scale", "rf_quotient_probe"]
+           "rf_mlp_calibrate_scale", "rf_quotient_probe", "rf_volume_fusion_lists"]
 
 
 def _load():
@@ -178,6 +178,7 @@ def _load():
         "rf_learned_step": (i, [P, P, i, ctypes.POINTER(rf_intrinsics), i, ctypes.POINTER(rf_pose), P, P, P]),
         "rf_l2_gather_probe": (i, [P, ctypes.c_size_t, i, i, i, P, P]),
         "rf_volume_counters": (i, [P, ctypes.POINTER(ctypes.c_longlong), i]),
+        "rf_volume_fusion_lists": (i, [P, ctypes.POINTER(ctypes.c_int)]),
         "rf_quotient_probe": (i, [P, P, ctypes.c_size_t, P, P]),
     }
     for name, (res, args) in sig.items():
@@ -315,6 +316,12 @@ class Volume:
         out = (ctypes.c_longlong * 3)()
         _check(lib.rf_volume_counters(self.handle, out, int(bool(reset))))
         return dict(voxels_updated=out[0], bricks_visited=out[1], bricks_repacked=out[2])
+
+    def fusion_lists(self):
+        """rf_volume_fusion_lists: (bricks projected voxel by voxel, bricks fused as free space) of the last fusion."""
+        out = (ctypes.c_int * 2)()
+        _check(lib.rf_volume_fusion_lists(self.handle, out))
+        return out[0], out[1]
 
     def upload(self, codes: np.ndarray, weights: np.ndarray | None = None):
         """codes: storage codes, shape (dz, dy, dx) or flat x-fastest."""

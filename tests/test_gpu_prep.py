@@ -188,14 +188,16 @@ def test_integrate_parity_many_bricks(oracle, nat):
 @pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
 def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
     """Volumes on both sides of the brick count from which whole bricks are fused as free space, a frame that ends
-    inside a pixel tile and has holes, and a map that already holds weights up to their limit, unobserved voxels and
-    values other than +1 in front of the surface: values and weights against the oracle after three frames."""
+    inside a pixel tile, with unequal focal lengths and clustered holes, and a map that already holds weights up to
+    their limit, unobserved voxels and values other than +1 in front of the surface: values and weights against the
+    oracle after three frames, in which many bricks of the large map went the free-space way."""
     import torch
 
     voxel, trunc = 5.12 / max(dims), 4 * 5.12 / max(dims)
     scene = synth.make_scene(5.12, 0.3, 11)
     traj = synth.make_trajectory(scene, 3, 2.0, 2.0, 11)
-    K = synth.intrinsics(97, 61)
+    K = synth.intrinsics(197, 131)
+    K["fy"] *= 1.2
     rng = np.random.default_rng(3)
     shape = dims[::-1]
     F0 = np.where(rng.random(shape) < 0.02, rng.uniform(-1, 1, shape), 1.0)
@@ -210,11 +212,14 @@ def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
     amb = np.zeros(F0.size, bool)
     for f in range(3):
         depth = synth.render_depth(scene, traj[f], K, rng)
-        depth[rng.random(depth.shape) < 0.003] = 0.0
+        depth[20:37, 60:90] = 0.0
+        depth[100:, 150:][rng.random((31, 47)) < 0.1] = np.nan
         pose = traj[f].astype(np.float32).astype(np.float64)
         amb |= ov.integrate_ambiguity(depth, K, pose, tol=1e-4).astype(bool)
         ov.integrate(depth, K, pose, threads=8)
         nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
+        projected, free = gv.fusion_lists()
+        assert projected > 100 and (free > 100 if np.prod(dims) // 512 >= 16384 else free == 0)
     codes, W = gv.download()
     Fg = synth.decode_values(codes).reshape(-1)
     sure = ~amb
@@ -250,6 +255,7 @@ def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
         amb |= ov.integrate_ambiguity(depth, K, pose, tol=1e-4).astype(bool)
         ov.integrate(depth, K, pose, threads=8)
         nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
+        assert (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 16384)
     codes, W = gv.download()
     Fg = synth.decode_values(codes).reshape(-1)
     sure = ~amb
@@ -282,6 +288,7 @@ def test_integrate_keeps_infinities(nat, dtype, dims):
     depth = np.full((120, 160), 8.5, np.float32)  # beyond the map: f = 1 in every voxel in view
     depth[50:60, 70:75] = 0.0
     nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, [1, 0, 0, 0, 2.5, 2.5, -1.0])
+    assert gv.fusion_lists()[0] > 20 and (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 16384)
     F1, W1 = gv.download()
     F1, W1 = F1.reshape(shape), W1.reshape(shape)
     up = W1 == W0 + 1
