@@ -53,7 +53,7 @@ rf_status rf_volume_counters(rf_volume v, long long out_host[3], int reset);
 /*
  * rf_volume_fusion_lists -- how the last tsdf_integrate took the bricks that passed
  * its frustum test: out_host[0] projected voxel by voxel, out_host[1] fused as free
- * space as a whole (volumes of 16,384 bricks and more).  Synchronises the device.
+ * space as a whole (volumes of 49,152 bricks and more).  Synchronises the device.
  */
 rf_status rf_volume_fusion_lists(rf_volume v, int out_host[2]);
 

@@ -185,7 +185,7 @@ def test_integrate_parity_many_bricks(oracle, nat):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f16", "i16"])
-@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+@pytest.mark.parametrize("dims", [(304, 296, 288), (96, 104, 88)])
 def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
     """Volumes on both sides of the brick count from which whole bricks are fused as free space, a frame that ends
     inside a pixel tile, with unequal focal lengths and clustered holes, and a map that already holds weights up to
@@ -219,7 +219,7 @@ def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
         ov.integrate(depth, K, pose, threads=8)
         nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
         projected, free = gv.fusion_lists()
-        assert projected > 100 and (free > 100 if np.prod(dims) // 512 >= 16384 else free == 0)
+        assert projected > 100 and (free > 100 if np.prod(dims) // 512 >= 49152 else free == 0)
     codes, W = gv.download()
     Fg = synth.decode_values(codes).reshape(-1)
     sure = ~amb
@@ -233,7 +233,7 @@ def test_integrate_free_space_bricks(oracle, nat, dtype, dims):
 
 
 @pytest.mark.parametrize("sx,sy", [(1, -1), (-1, 1), (-1, -1)])
-@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+@pytest.mark.parametrize("dims", [(304, 296, 288), (96, 104, 88)])
 def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
     """A focal length may have either sign (some datasets publish fy = -480): a fresh map on both sides of the brick
     count from which whole bricks are fused as free space, unequal focal lengths, two frames, against the oracle."""
@@ -255,7 +255,7 @@ def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
         amb |= ov.integrate_ambiguity(depth, K, pose, tol=1e-4).astype(bool)
         ov.integrate(depth, K, pose, threads=8)
         nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, pose)
-        assert (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 16384)
+        assert (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 49152)
     codes, W = gv.download()
     Fg = synth.decode_values(codes).reshape(-1)
     sure = ~amb
@@ -267,7 +267,7 @@ def test_integrate_negative_focal_length(oracle, nat, dims, sx, sy):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
-@pytest.mark.parametrize("dims", [(208, 216, 200), (96, 104, 88)])
+@pytest.mark.parametrize("dims", [(304, 296, 288), (96, 104, 88)])
 def test_integrate_keeps_infinities(nat, dtype, dims):
     """Values that a float or half map can hold but no frame produces: the running average (W F + 1) / (W + 1) as IEEE
     arithmetic gives it, in free bricks, in bricks next to invalid pixels and on small maps."""
@@ -288,7 +288,7 @@ def test_integrate_keeps_infinities(nat, dtype, dims):
     depth = np.full((120, 160), 8.5, np.float32)  # beyond the map: f = 1 in every voxel in view
     depth[50:60, 70:75] = 0.0
     nat.tsdf_integrate(gv, torch.from_numpy(depth).cuda(), K, [1, 0, 0, 0, 2.5, 2.5, -1.0])
-    assert gv.fusion_lists()[0] > 20 and (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 16384)
+    assert gv.fusion_lists()[0] > 20 and (gv.fusion_lists()[1] > 100) == (np.prod(dims) // 512 >= 49152)
     F1, W1 = gv.download()
     F1, W1 = F1.reshape(shape), W1.reshape(shape)
     up = W1 == W0 + 1
