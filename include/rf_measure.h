@@ -1,7 +1,7 @@
 /*
  * rf_measure.h -- measurement entry points of librosefusion.so.  They serve the
- * roofline statements about the hot path; the paper has no counterpart for
- * either (it reports only frame rates and per-frame times).  The general rules
+ * roofline statements about the hot path and the tests of its parts; the paper has no
+ * counterpart for them (it reports only frame rates and per-frame times).  The general rules
  * of rosefusion.h apply (status codes, *_dev device pointers, streams).
  */
 #ifndef RF_MEASURE_H

@@ -77,7 +77,10 @@ void rf_mlp_destroy(rf_mlp m);
 rf_status rf_mlp_set_params(rf_mlp m, const float *theta_host);
 rf_status rf_mlp_get_params(rf_mlp m, float *theta_host);
 /*
- * rf_mlp_forward -- o for `batch` input rows.
+ * rf_mlp_forward -- o for `batch` input rows.  Up to 8 rows and 9 or more are summed
+ * in different orders, so the same row's outputs agree to FP32 rounding between the
+ * two (and, where a hidden value lies next to a rounding boundary, to one bfloat16
+ * step of it), not bit for bit; within either they do not depend on the batch.
  *   x_dev    device uint16[batch * RF_MLP_IN] (bfloat16 bit patterns), row-major
  *   out_dev  device float[batch * RF_MLP_OUT]
  */

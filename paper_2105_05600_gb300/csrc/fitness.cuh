@@ -359,7 +359,7 @@ __host__ __device__ inline Split make_split(int n, int m, int total_warps, int m
     int want = (UNITS_PER_WARP * total_warps + g32 - 1) / g32;
     int lo = (m + CHUNK_MAX - 1) / CHUNK_MAX;   // staging capacity
     int hi = (m + MIN_CHUNK - 1) / MIN_CHUNK;   // at least MIN_CHUNK points per unit
-    if (s.groups * hi < total_warps)  // (1024 particles x 4800 points: 582 -> 536 us a frame)
+    if (s.groups * hi < total_warps)  // (1024 particles x 4800 points: 555 -> 521 us a frame)
         hi = (m + SMALL_CHUNK - 1) / SMALL_CHUNK;
     want = want < lo ? lo : want;
     want = want > hi ? hi : want;

@@ -4,9 +4,12 @@
 // frame (the c_0, r_0 of the Sec. 4 initialisation).  Training (forward, loss,
 // backward, Adam) and inference run only the kernels of this file.
 //
-// Every product is one launch of umma_gemm_kernel:
+// Forward passes of up to 8 rows are one launch of forward_small_kernel.  Every other
+// product is a part of a launch of umma_gemm_kernel:
 //     C[M x N] = A[M x K] . B[N x K]^T,  A, B bfloat16 row-major (K contiguous),
 //     FP32 accumulation in tensor memory (TMEM), fused epilogue.
+// A forward layer is a launch of its own; a backward launch holds a layer's weight and
+// input gradients and its bias gradient (the first one also the total of the loss).
 // One CTA owns a 128 x 32 tile of C and 32 TMEM columns:
 //   warp 0, lane 0   TMA producer: 64-column slabs of A (128 rows) and B (32 rows)
 //                    into a 5-stage shared-memory ring (mbarrier transaction
@@ -28,7 +31,7 @@
 // 219 / 38 / 41, N 64: 170 / 30 / 35, N 32: 150 / 29 / 44, N 16: 135 / 27 / 68.  Five
 // stages rather than eight leave room for two CTAs on an SM, so that the next launch of a
 // chain can set up beside this one; with that and its operands of the epilogue fetched
-// before the products are done, a forward pass takes 23 us at 1 row and 27 at 4096.
+// before the products are done, a forward pass takes 21 us at 9 rows and 26 at 4096.
 // Shared-memory operand layout: K-major with the 128-byte swizzle that TMA writes and
 // the MMA reads -- a slab row is 128 bytes, eight rows are one 1024-byte atom, so the
 // stride-dimension (M/N) byte offset is 1024, the leading-dimension offset is unused,
@@ -498,8 +501,9 @@ __global__ void __launch_bounds__(GB_THREADS, 2) umma_gemm_kernel(const __grid_c
 // bfloat16 as the products' epilogue does and written to all CTAs' shared memory between
 // cluster barriers.  Bound by latency: four dependent layers of a load, a sum and a
 // barrier, and one row's sums after another's.  Against the four chained products:
-// 4.4 instead of about 21 us of device time at 1 row (8.8 : 22.6 with the launches),
-// 12.3 : 22.6 at 8 rows; a row more costs 1.1 us, so the line is drawn at 8.
+// 6.4 : 20.7 us back to back at 1 row (4.4 of device time), 12.4 : 20.7 at 8.  A row more
+// costs 0.9 us, so the two would meet near 16 rows; 8 is as many as a frame or a last batch
+// asks for with rows and activations in 26 KB of static shared memory (16 need 51 of 48).
 constexpr int SMALL_BATCH = 8, SMALL_CTAS = 8, SMALL_THREADS = 512;
 constexpr int SMALL_PIECES = (RF_MLP_IN / 8 + 31) / 32;  // 16-byte pieces of a first-layer row per lane
 static_assert(SMALL_CTAS * SMALL_THREADS / 32 * 2 == RF_MLP_HIDDEN && RF_MLP_HIDDEN == 256, "two outputs per warp");
