@@ -315,10 +315,12 @@ def test_tracker_is_deterministic(oracle, nat):
     assert out[0][1] == out[1][1]
 
 
-# a remainder of a block of 512 ordered particles, two whole blocks, one particle over, a remainder of a warp
-@pytest.mark.parametrize("n", [874, 1024, 1025, 2100])
-def test_tracker_parity_ordered_swarm(oracle, nat, n):
-    """Frames of 160 x 120 points, from 2^24 lookups an iteration, whose swarm is scored in an order of its own."""
+# a remainder of a block of 512 ordered particles, two whole blocks, one particle over, a remainder of a warp, more
+# blocks than the half of the grid that orders them
+@pytest.mark.parametrize("n,w,h", [(874, 160, 120), (1024, 160, 120), (1025, 160, 120), (2100, 160, 120),
+                                   (100003, 16, 12)])
+def test_tracker_parity_ordered_swarm(oracle, nat, n, w, h):
+    """Frames from 2^24 lookups an iteration, whose swarm is scored in an order of its own."""
     import torch
 
     scene, codes, F64, cfg = analytic_volume_codes("tiny", dtype="i16")
@@ -326,10 +328,10 @@ def test_tracker_parity_ordered_swarm(oracle, nat, n):
     gv.upload(codes)
     ov = oracle_volume(oracle, cfg, F64)
     traj = synth.make_trajectory(scene, 2, cfg["speed"], cfg["ang_speed"], cfg["seed"])
-    K = synth.intrinsics(160, 120)
+    K = synth.intrinsics(w, h)
     d0, d1 = (synth.render_depth(scene, traj[f], K) for f in range(2))
-    assert n * 160 * 120 >= 1 << 24
-    tr = nat.Tracker(gv, nat.pst_create(n, seed=1), nat.make_params(k_max=3), 160, 120)
+    assert n * w * h >= 1 << 24
+    tr = nat.Tracker(gv, nat.pst_create(n, seed=1), nat.make_params(k_max=3), w, h)
     tr.set_scale([0.1] * 6)
     prev = pose_f32(traj[0])
     pose, gst, status = nat.pfo_track_frame(tr, torch.from_numpy(d1).cuda(), torch.from_numpy(d0).cuda(), K, prev)
